@@ -11,8 +11,8 @@
 //      element once, instead of once per output tile that reads it.
 //   2. GEMM: a persistent warp-specialised tcgen05 kernel.  One TMA warp
 //      streams 128x64 A and 256x64 W tiles (one 64-wide quantization group
-//      per stage, 64-byte swizzle) into an 8-stage shared-memory ring and
-//      each group's scales into a ring of its own; one thread issues
+//      per stage, 64-byte swizzle) into a 6-stage shared-memory ring, with
+//      each group's scales on the same barrier; one thread issues
 //      kind::f8f6f4 MMAs into a fresh fp32 TMEM accumulator for every group
 //      (double-buffered, 2 x 256 columns), so each accumulator holds exactly
 //      P_g = sum_{k in g} v_a v_w; sixteen epilogue warps read P_g with
@@ -219,22 +219,32 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constan
 constexpr int BM = 128;
 constexpr int BN = 256;
 constexpr int BK = kGroupQ;
-constexpr int kStages = 8;
 constexpr int kABytes = BM * BK;      // E4M3 operands: one byte per element
 constexpr int kBBytes = BN * BK;
 constexpr int kStageBytes = kABytes + kBBytes;
 // Warpgroups 0-3 dequantise (16 warps: four per 32-lane TMEM quarter, 64
-// columns each); warpgroup 4 holds the operand TMA producer, the MMA issuer,
-// the scale copier and one idle warp.  The dequant epilogue is the
-// throughput-critical part (two fp32 operations per output element per
-// group), so it gets four warps per scheduler; the three control roles sit on
-// three different schedulers (warp w runs on scheduler w % 4) because each
-// slows the epilogue warps that share its scheduler.
+// columns each); warpgroup 4 holds the TMA producer, the MMA issuer and two
+// idle warps.  The dequant epilogue is the throughput-critical part (two fp32
+// operations per output element per group), so it gets four warps per
+// scheduler; the control roles sit on two different schedulers (warp w runs
+// on scheduler w % 4) because each slows the epilogue warps that share its
+// scheduler.
+//
+// What bounds the kernel is the time each epilogue warp spends per group
+// outside its arithmetic: TMEM and shared loads and the hand-off.  So a group
+// costs an epilogue warp one barrier wait and one arrival (its scales ride on
+// the operands' barrier, see Smem), waits branch on a warp vote
+// (mbar_wait_warp) and the control warps run their loops converged with one
+// elected lane issuing, which took an operand stage's issue from about 460 to
+// 60 cycles.  Together, against single-lane control loops, per-lane waits and
+// a scale ring with barriers of its own (CUDA events, GEMM + combine):
+// 18432 x 12288 x 3072 1178 -> 1053 us, 8192 x 4608 x 1152 96.9 -> 86.7,
+// 2048 x 4096 x 11008 (E5M2) 166.6 -> 150.2; per-row scales 18432 x 3072 x
+// 3072 251 -> 181, asymmetric 548 -> 478.
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 4) * 32;
 constexpr int kProducerWarp = kEpiWarps;
 constexpr int kMmaWarp = kEpiWarps + 1;
-constexpr int kSideWarp = kEpiWarps + 2;
 constexpr int kColsPerWarp = BN / 4;
 // Register split (setmaxnreg): 640 threads launch with 96 registers each;
 // warpgroup 4 drops to 32 so the epilogue warpgroups can hold 112
@@ -285,18 +295,25 @@ struct GemmArgs {
 };
 
 // Shared memory: the operand stages, then a ring of side-value slots (one
-// group's NSIDE x BM activation and NSIDE x BN weight values each, copied by
-// the producer and released by the epilogue), then the mbarriers.
+// group's NSIDE x BM activation and NSIDE x BN weight values each), then the
+// mbarriers.  6 stages cover the copy latency (a group takes 350 cycles or
+// more); 5 and 8 measured 1% slower.  A group's side values are copied with
+// its operands and counted on the same barrier.  A slot needs no barrier of its own to be reused: the
+// producer writes group i + kSideSlots once the MMA of group i + kSideSlots -
+// kStages is done, which was issued after the epilogue had released group
+// i + kSideSlots - kStages - 2, a group after i.
 template <int NSIDE>
 struct Smem {
+    static constexpr int kStages = NSIDE == 1 ? 6 : 5;
+    static constexpr int kSideSlots = NSIDE == 1 ? 16 : 8;
+    static_assert(kSideSlots >= kStages + 3, "a slot is rewritten only after its group's epilogue");
     static constexpr int kOperands = 0;
     static constexpr int kSide = kStages * kStageBytes;
-    static constexpr int kSideSlots = NSIDE == 1 ? 8 : 4;
     static constexpr int kSideABytes = NSIDE * BM * 4;
     static constexpr int kSideSlotBytes = NSIDE * (BM + BN) * 4;
     static constexpr int kBars = kSide + kSideSlots * kSideSlotBytes;
-    // full, empty, acc_full x2, acc_empty x2, drain, side_full, side_empty
-    static constexpr int kNumBars = 2 * kStages + 4 + 1 + 2 * kSideSlots;
+    // full, empty, acc_full x2, acc_empty x2, drain
+    static constexpr int kNumBars = 2 * kStages + 4 + 1;
     static constexpr int kMisc = kBars + kNumBars * 8;
     static constexpr int kTotal = kMisc + 16;
     static constexpr int kAlloc = kTotal + 1024;  // slack to align the base to 1024 bytes
@@ -546,6 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     griddep_wait();
     constexpr int NSIDE = (MODE == QUARTZ_ASYMMETRIC) ? 3 : 1;
     using L = Smem<NSIDE>;
+    constexpr int kStages = L::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
@@ -558,8 +576,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto acc_full_bar = [&](int b) { return bar_base + 8u * (2 * kStages + b); };
     auto acc_empty_bar = [&](int b) { return bar_base + 8u * (2 * kStages + 2 + b); };
     const uint32_t drain_bar = bar_base + 8u * (2 * kStages + 4);
-    auto side_full_bar = [&](int s) { return bar_base + 8u * (2 * kStages + 5 + s); };
-    auto side_empty_bar = [&](int s) { return bar_base + 8u * (2 * kStages + 5 + L::kSideSlots + s); };
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + L::kMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kMisc + 4);
 
@@ -569,14 +585,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(acc_full_bar(b), 1);
+            mbar_init(acc_full_bar(b), 2);  // the commit and the issuing lane
             mbar_init(acc_empty_bar(b), kEpiWarps);
         }
         mbar_init(drain_bar, 1);
-        for (int s = 0; s < L::kSideSlots; ++s) {
-            mbar_init(side_full_bar(s), 1);
-            mbar_init(side_empty_bar(s), kEpiWarps);
-        }
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -600,77 +612,57 @@ __global__ void __launch_bounds__(kThreads, 1)
         // ------------------------------------------------------------------
         // TMA producer: one stage = one 64-wide group of A (128 rows) and W
         // (256 rows).  Rows past M or N are zero-filled by the tensor map.
+        // The whole warp runs the loop and one elected lane issues (see
+        // elect_one): a stage costs about 60 cycles this way, against 460
+        // from a divergent lane.
         // ------------------------------------------------------------------
-        if (lane == 0) {
-            int it = 0;  // groups whose operand copies were issued
-            bool ok = true;
-            const int n_items = work_items(args);
-            for (int k = 0; k < n_items && ok; ++k) {
-                const WorkItem wi = work_item(args, k);
-                int mt, nt;
-                tile_coords<RM>(wi.tile, args, mt, nt);
-                for (int g = wi.g0; g < wi.g1; ++g, ++it) {
-                    const int s = it % kStages;
-                    if (it >= kStages &&
-                        !mbar_wait_bounded(empty_bar(s), ((it / kStages) - 1) & 1, abort_flag,
-                                           args.dev_err, kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
+        const bool leader = elect_one();
+        const int64_t a_plane = args.m_pad * G, w_plane = args.n_pad * G;
+        int it = 0, s = 0;   // groups whose operand copies were issued; the next stage
+        uint32_t phase = 1;  // parity of that stage's last release (the first round waits for none)
+        bool ok = true;
+        const int n_items = work_items(args);
+        for (int k = 0; k < n_items && ok; ++k) {
+            const WorkItem wi = work_item(args, k);
+            int mt, nt;
+            tile_coords<RM>(wi.tile, args, mt, nt);
+            const float *src_a = args.a_side + wi.g0 * args.m_pad + static_cast<int64_t>(mt) * BM;
+            const float *src_w = args.w_side + wi.g0 * args.n_pad + static_cast<int64_t>(nt) * BN;
+            for (int g = wi.g0; g < wi.g1; ++g, ++it) {
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, args.dev_err, kWaitLimitNs)) {
+                    ok = false;
+                    break;
+                }
+                if (leader) {
                     const uint32_t sa = smem_base + L::kOperands + s * kStageBytes;
-                    mbar_arrive_expect_tx(full_bar(s), kStageBytes);
+                    mbar_arrive_expect_tx(full_bar(s), kStageBytes + (PERROW ? 0 : L::kSideSlotBytes));
                     tma_load_2d(sa, &tmap_a, g * BK, mt * BM, full_bar(s));
                     tma_load_2d(sa + kABytes, &tmap_w, g * BK, nt * BN, full_bar(s));
+                    if (!PERROW) {
+                        const uint32_t dst = smem_base + L::kSide + (it % L::kSideSlots) * L::kSideSlotBytes;
+#pragma unroll
+                        for (int sd = 0; sd < NSIDE; ++sd) {
+                            bulk_load(dst + sd * BM * 4, src_a + sd * a_plane, BM * 4, full_bar(s));
+                            bulk_load(dst + L::kSideABytes + sd * BN * 4, src_w + sd * w_plane, BN * 4, full_bar(s));
+                        }
+                    }
                 }
-            }
-            // Never leave the CTA with copies in flight: wait for the last
-            // load issued into every stage (bounded, even after an abort).
-            int zero = 0;
-            for (int s = 0; s < kStages && s < it; ++s) {
-                const int last = it - 1 - ((it - 1 - s) % kStages);
-                mbar_wait_bounded(full_bar(s), (last / kStages) & 1, &zero, args.dev_err, kWaitLimitNs);
+                __syncwarp();
+                src_a += args.m_pad;
+                src_w += args.n_pad;
+                if (++s == kStages) {
+                    s = 0;
+                    phase ^= 1u;
+                }
             }
         }
-        __syncwarp();
-      } else if (warp == kSideWarp) {
-        // ------------------------------------------------------------------
-        // Scale copier: each group's side values (scales; asymmetric also
-        // zero-point terms) go by bulk copy into a ring slot that the
-        // epilogue frees.
-        // ------------------------------------------------------------------
-        if (!PERROW && lane == 0) {
-            constexpr int S = L::kSideSlots;
-            const int64_t a_plane = args.m_pad * G;
-            const int64_t w_plane = args.n_pad * G;
-            int it = 0;  // groups whose side-value copies were issued
-            bool ok = true;
-            const int n_items = work_items(args);
-            for (int k = 0; k < n_items && ok; ++k) {
-                const WorkItem wi = work_item(args, k);
-                int mt, nt;
-                tile_coords<RM>(wi.tile, args, mt, nt);
-                for (int g = wi.g0; g < wi.g1; ++g, ++it) {
-                    const int ss = it % S;
-                    if (it >= S && !mbar_wait_bounded(side_empty_bar(ss), ((it / S) - 1) & 1, abort_flag,
-                                                      args.dev_err, kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t dst = smem_base + L::kSide + ss * L::kSideSlotBytes;
-                    mbar_arrive_expect_tx(side_full_bar(ss), L::kSideSlotBytes);
-                    const float *src_a = args.a_side + static_cast<int64_t>(g) * args.m_pad + static_cast<int64_t>(mt) * BM;
-                    const float *src_w = args.w_side + static_cast<int64_t>(g) * args.n_pad + static_cast<int64_t>(nt) * BN;
-#pragma unroll
-                    for (int sd = 0; sd < NSIDE; ++sd) {
-                        bulk_load(dst + sd * BM * 4, src_a + sd * a_plane, BM * 4, side_full_bar(ss));
-                        bulk_load(dst + L::kSideABytes + sd * BN * 4, src_w + sd * w_plane, BN * 4, side_full_bar(ss));
-                    }
-                }
-            }
+        // Never leave the CTA with copies in flight: wait for the last
+        // load issued into every stage (bounded, even after an abort).
+        if (leader) {
             int zero = 0;
-            for (int s = 0; s < S && s < it; ++s) {
-                const int last = it - 1 - ((it - 1 - s) % S);
-                mbar_wait_bounded(side_full_bar(s), (last / S) & 1, &zero, args.dev_err, kWaitLimitNs);
+            for (int i = 0; i < kStages && i < it; ++i) {
+                const int last = it - 1 - ((it - 1 - i) % kStages);
+                mbar_wait_bounded(full_bar(i), (last / kStages) & 1, &zero, args.dev_err, kWaitLimitNs);
             }
         }
         __syncwarp();
@@ -680,50 +672,56 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a fresh accumulator (first MMA overwrites), then two commits: one
         // frees the operand stage, one hands P_g to the epilogue.
         // ------------------------------------------------------------------
-        if (lane == 0) {
+        {
             const uint32_t idesc = args.wide ? idesc_e5m2_f32(BM, BN) : idesc_e4m3_f32(BM, BN);
-            int it = 0;
+            const uint64_t desc_a0 = sdesc_k_major_sw64(smem_base + L::kOperands);
+            const uint64_t desc_w0 = sdesc_k_major_sw64(smem_base + L::kOperands + kABytes);
+            const bool leader = elect_one();
+            int s = 0;
+            uint32_t phase = 0;
             bool ok = true;
             constexpr int CH = PERROW ? kPerRowChunk : 1;  // stages per TMEM accumulator
             int ic = 0;                                    // accumulators handed to the epilogue
             const int n_items = work_items(args);
             for (int k = 0; k < n_items && ok; ++k) {
                 const WorkItem wi = work_item(args, k);
-                for (int g = wi.g0; g < wi.g1; ++g, ++it) {
-                    const int s = it % kStages;
+                for (int g = wi.g0; g < wi.g1; ++g) {
                     const int b = ic & 1;
                     const bool first = (g % CH) == 0;
                     const bool last = (g % CH) == CH - 1 || g == G - 1;
-                    if (!mbar_wait_bounded(full_bar(s), (it / kStages) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
-                    if (first && ic >= 2 && !mbar_wait_bounded(acc_empty_bar(b), ((ic >> 1) - 1) & 1,
-                                                               abort_flag, args.dev_err, kWaitLimitNs)) {
+                    if (!mbar_wait_warp(full_bar(s), phase, abort_flag, args.dev_err, kWaitLimitNs) ||
+                        (first && ic >= 2 && !mbar_wait_warp(acc_empty_bar(b), ((ic >> 1) - 1) & 1, abort_flag,
+                                                             args.dev_err, kWaitLimitNs))) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_base + L::kOperands + s * kStageBytes;
-                    const uint32_t d = tmem_base + static_cast<uint32_t>(b * BN);
+                    const uint64_t st = static_cast<uint64_t>(s * (kStageBytes / 16));  // (descriptor address units)
+                    if (leader) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 32; ++kk) {
-                        const uint64_t adesc = sdesc_k_major_sw64(sa + kk * 32);
-                        const uint64_t bdesc = sdesc_k_major_sw64(sa + kABytes + kk * 32);
-                        mma_f8_ss(d, adesc, bdesc, idesc, (kk > 0 || !first) ? 1u : 0u);
+                        for (int kk = 0; kk < BK / 32; ++kk)
+                            mma_f8_ss(tmem_base + static_cast<uint32_t>(b * BN), desc_a0 + st + 2 * kk,
+                                      desc_w0 + st + 2 * kk, idesc, (kk > 0 || !first) ? 1u : 0u);
+                        mma_commit(empty_bar(s));
+                        if (last) {
+                            mma_commit(acc_full_bar(b));
+                            mbar_arrive(acc_full_bar(b));  // orders the side values, seen landed above, before their readers
+                        }
                     }
-                    mma_commit(empty_bar(s));
-                    if (last) {
-                        mma_commit(acc_full_bar(b));
-                        ++ic;
+                    __syncwarp();
+                    if (last) ++ic;
+                    if (++s == kStages) {
+                        s = 0;
+                        phase ^= 1u;
                     }
                 }
             }
             // Make sure no MMA is still writing TMEM before it is freed.
-            mma_commit(drain_bar);
-            int zero = 0;
-            mbar_wait_bounded(drain_bar, 0, &zero, args.dev_err, kWaitLimitNs);
+            if (leader) {
+                mma_commit(drain_bar);
+                int zero = 0;
+                mbar_wait_bounded(drain_bar, 0, &zero, args.dev_err, kWaitLimitNs);
+            }
         }
         __syncwarp();
       }
@@ -768,8 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int j = 0; j < 16; ++j) acci[c][j] = 0;
                 for (int cc = 0; cc < nchunks; ++cc, ++ic) {
                     const int b = ic & 1;
-                    if (!mbar_wait_bounded(acc_full_bar(b), (ic >> 1) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
+                    if (!mbar_wait_warp(acc_full_bar(b), (ic >> 1) & 1, abort_flag, args.dev_err, kWaitLimitNs)) {
                         ok = false;
                         break;
                     }
@@ -839,16 +836,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int g = wi.g0; g < wi.g1; ++g, ++it) {
                     const int b = it & 1;
                     const int ss = it % S;
-                    if (!mbar_wait_bounded(side_full_bar(ss), (it / S) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
                     const uint32_t side_a = smem_base + L::kSide + ss * L::kSideSlotBytes + (quarter * 32 + 4 * trow) * 4;
                     const uint32_t side_w = smem_base + L::kSide + ss * L::kSideSlotBytes + L::kSideABytes +
                                             (slot * kColsPerWarp + tq) * 4;
-                    if (!mbar_wait_bounded(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
+                    if (!mbar_wait_warp(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err, kWaitLimitNs)) {
                         ok = false;
                         break;
                     }
@@ -865,10 +856,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(acc_empty_bar(b));
-                        mbar_arrive(side_empty_bar(ss));
-                    }
+                    if (lane == 0) mbar_arrive(acc_empty_bar(b));
                 }
                 if (!ok) break;
                 if (wi.part >= 0) {
@@ -901,16 +889,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int g = 0; g < G; ++g, ++it) {
                     const int b = it & 1;
                     const int ss = it % S;
-                    if (!mbar_wait_bounded(side_full_bar(ss), (it / S) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
                     const uint32_t side_a = smem_base + L::kSide + ss * L::kSideSlotBytes + (quarter * 32 + 4 * trow) * 4;
                     const uint32_t side_w = smem_base + L::kSide + ss * L::kSideSlotBytes + L::kSideABytes +
                                             (slot * kColsPerWarp + tq) * 4;
-                    if (!mbar_wait_bounded(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err,
-                                           kWaitLimitNs)) {
+                    if (!mbar_wait_warp(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err, kWaitLimitNs)) {
                         ok = false;
                         break;
                     }
@@ -970,10 +952,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(acc_empty_bar(b));
-                        mbar_arrive(side_empty_bar(ss));
-                    }
+                    if (lane == 0) mbar_arrive(acc_empty_bar(b));
                 }
                 if (!ok) break;
                 int mt, nt;

@@ -25,6 +25,20 @@ __device__ __forceinline__ float4 lds_f4(uint32_t addr)
     return v;
 }
 
+// True in one lane of a converged warp.  A warp whose lanes all run a loop and
+// whose elected lane issues the copies or MMAs keeps their operands (barrier
+// and descriptor addresses) warp-uniform.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ uint64_t global_timer_ns()
 {
     uint64_t t;
@@ -104,6 +118,31 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
             return false;
         }
     }
+}
+
+// mbar_wait_bounded for a converged warp: every decision is a warp vote, so
+// the branches are uniform (a per-lane return from the loop costs a ready
+// wait about 75 cycles of reconvergence: 120 against 45 cycles measured).
+__device__ __forceinline__ bool mbar_wait_warp_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                    int *dev_err, uint64_t limit_ns)
+{
+    const uint64_t t0 = global_timer_ns();
+    for (;;) {
+        if (__all_sync(0xffffffffu, mbar_try_wait_sleep(bar, parity, 100000u))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        if (__any_sync(0xffffffffu, global_timer_ns() - t0 > limit_ns)) {
+            *abort_flag = 1;
+            atomicExch(dev_err, QUARTZ_DEV_TIMEOUT);
+            return false;
+        }
+    }
+}
+
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *dev_err,
+                                               uint64_t limit_ns)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return mbar_wait_warp_slow(bar, parity, abort_flag, dev_err, limit_ns);
 }
 
 // ---------------------------------------------------------------------------
