@@ -11,7 +11,7 @@
 //      element once, instead of once per output tile that reads it.
 //   2. GEMM: a persistent warp-specialised tcgen05 kernel.  One TMA warp
 //      streams 128x64 A and 256x64 W tiles (one 64-wide quantization group
-//      per stage, 64-byte swizzle) into a 6-stage shared-memory ring, with
+//      per stage, 64-byte swizzle) into a 5-stage shared-memory ring, with
 //      each group's scales on the same barrier; one thread issues
 //      kind::f8f6f4 MMAs into a fresh fp32 TMEM accumulator for every group
 //      (double-buffered, 2 x 256 columns), so each accumulator holds exactly
@@ -294,21 +294,24 @@ struct GemmArgs {
     float *tail_part;     // [tail_tiles][split][16][kEpiWarps * 32] float4 (fp32 pairs)
 };
 
-// Shared memory: the operand stages, then a ring of side-value slots (one
-// group's NSIDE x BM activation and NSIDE x BN weight values each), then the
-// mbarriers.  6 stages cover the copy latency (a group takes 350 cycles or
-// more); 5 and 8 measured 1% slower.  A group's side values are copied with
-// its operands and counted on the same barrier.  A slot needs no barrier of its own to be reused: the
+// Shared memory: the operand stages, the output blocks (one per epilogue warp,
+// see TileOut), then a ring of side-value slots (one group's NSIDE x BM
+// activation and NSIDE x BN weight values each), then the mbarriers.  5
+// stages cover the copy latency (a group takes 350 cycles or more; 4, 6 and 8
+// measured no better).  A group's side values are copied with its operands and counted
+// on the same barrier.  A slot needs no barrier of its own to be reused: the
 // producer writes group i + kSideSlots once the MMA of group i + kSideSlots -
 // kStages is done, which was issued after the epilogue had released group
 // i + kSideSlots - kStages - 2, a group after i.
-template <int NSIDE>
+constexpr int kOutBlockBytes = 32 * 128;  // 32 rows of 64 two-byte outputs
+template <int NSIDE, bool STAGED>
 struct Smem {
-    static constexpr int kStages = NSIDE == 1 ? 6 : 5;
+    static constexpr int kStages = 5;
     static constexpr int kSideSlots = NSIDE == 1 ? 16 : 8;
     static_assert(kSideSlots >= kStages + 3, "a slot is rewritten only after its group's epilogue");
     static constexpr int kOperands = 0;
-    static constexpr int kSide = kStages * kStageBytes;
+    static constexpr int kOut = kStages * kStageBytes;
+    static constexpr int kSide = kOut + (STAGED ? kEpiWarps * kOutBlockBytes : 0);
     static constexpr int kSideABytes = NSIDE * BM * 4;
     static constexpr int kSideSlotBytes = NSIDE * (BM + BN) * 4;
     static constexpr int kBars = kSide + kSideSlots * kSideSlotBytes;
@@ -402,20 +405,25 @@ __device__ __forceinline__ void add2_rn(uint64_t &a, uint64_t b)
     asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
 }
 
+// Two values rounded to a two-byte output type, the first in the low half.
+template <int OUT>
+__device__ __forceinline__ uint32_t pack2(float lo, float hi)
+{
+    if (OUT == QUARTZ_OUT_BF16) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(lo, hi);
+        return *reinterpret_cast<const uint32_t *>(&a);
+    }
+    const __half2 a = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&a);
+}
+
 template <int OUT>
 __device__ __forceinline__ void store_quad(void *y, int64_t off, float4 v)
 {
-    if (OUT == QUARTZ_OUT_F16) {
-        const __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
-        *reinterpret_cast<uint2 *>(static_cast<__half *>(y) + off) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
-    } else if (OUT == QUARTZ_OUT_BF16) {
-        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-        *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(y) + off) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
-    } else {
+    if (OUT == QUARTZ_OUT_F32)
         *reinterpret_cast<float4 *>(static_cast<float *>(y) + off) = v;
-    }
+    else
+        *reinterpret_cast<uint2 *>(static_cast<uint16_t *>(y) + off) = make_uint2(pack2<OUT>(v.x, v.y), pack2<OUT>(v.z, v.w));
 }
 
 // v + bias[n .. n + 3] in fp32 (no bias: v).
@@ -433,36 +441,73 @@ __device__ __forceinline__ float4 add_bias4(const GemmArgs &args, int64_t n, flo
     return v;
 }
 
-// Output of one 128 x 256 tile from the symmetric epilogue's registers:
-// acc[c][4h + i] holds output column 16c + tq + i of this warp's slice, rows
-// trow + 16h (low half) and trow + 16h + 8 (high half) of its quarter; the
-// bias is added in fp32, then one rounding to the output type.
-template <int OUT, int RM>
-__device__ __forceinline__ void store_tile_sym(const GemmArgs &args, int tile, int quarter, int slot, int trow,
-                                               int tq, const uint64_t (&acc)[4][8])
-{
-    int mt, nt;
-    tile_coords<RM>(tile, args, mt, nt);
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int64_t m = static_cast<int64_t>(mt) * BM + quarter * 32 + 16 * h + 8 * e + trow;
-            if (m >= args.M) continue;
-#pragma unroll
-            for (int chunk = 0; chunk < 4; ++chunk) {
-                const int64_t n = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + 16 * chunk + tq;
-                if (n >= args.N) continue;
-                float vv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint64_t q = acc[chunk][4 * h + i];
-                    vv[i] = __uint_as_float(static_cast<uint32_t>(e ? (q >> 32) : q));
-                }
-                store_quad<OUT>(args.y, m * args.N + n, add_bias4(args, n, make_float4(vv[0], vv[1], vv[2], vv[3])));
-            }
+// Output of one epilogue warp's 32 x 64 slice of a tile.  Two-byte outputs go
+// through the warp's block of shared memory (128-byte rows, 128-byte swizzle:
+// the 8-byte writes of a warp then hit every bank twice at most) and leave it
+// by one tensor store, which clips rows past M and columns past N, so that
+// the warp is back at its next group while the tile is written: with direct
+// 8-byte stores a tile held its warps for about 2 us.  fp32 outputs are
+// stored directly (their blocks would not fit).
+template <int OUT>
+struct TileOut {
+    static constexpr bool kStaged = OUT != QUARTZ_OUT_F32;
+    const GemmArgs &args;
+    const CUtensorMap *tmap;
+    uint32_t block, at;  // this warp's block; this thread's 8 bytes of a row, before row and chunk
+    uint32_t swz;
+    int64_t m0, n0;      // first row and column of the slice
+    int trow, tq, lane;
+
+    // (m, n): first row and column of the slice.  Made at the end of a tile,
+    // from a fresh read of the lane number, so that none of it takes
+    // registers in the group loop.
+    __device__ __forceinline__ TileOut(const GemmArgs &a, const CUtensorMap *t, uint32_t out_base, int warp, int64_t m,
+                                       int64_t n)
+        : args(a), tmap(t), m0(m), n0(n)
+    {
+        asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+        trow = lane >> 2;
+        tq = 4 * (lane & 3);
+        block = out_base + warp * kOutBlockBytes;
+        at = block + trow * 128 + ((2 * tq) & 15);
+        swz = static_cast<uint32_t>((trow ^ (tq >> 3)) << 4);
+        if (kStaged) {
+            if (lane == 0) bulk_wait_read();  // the previous tile has left the block
+            __syncwarp();
         }
-}
+    }
+
+    // v: columns 16 chunk + tq .. + 3 of row r8 + trow (r8: 0, 8, 16, 24) of
+    // the slice; the bias is added in fp32, then one rounding to the output
+    // type.
+    __device__ __forceinline__ void put(int r8, int chunk, float4 v)
+    {
+        const int64_t m = m0 + r8 + trow, n = n0 + 16 * chunk + tq;
+        if (n < args.N) v = add_bias4(args, n, v);
+        if (kStaged) {
+            sts_b64(at + r8 * 128 + ((32u * chunk) ^ swz), pack2<OUT>(v.x, v.y), pack2<OUT>(v.z, v.w));
+        } else if (m < args.M && n < args.N) {
+            *reinterpret_cast<float4 *>(static_cast<float *>(args.y) + m * args.N + n) = v;
+        }
+    }
+
+    __device__ __forceinline__ void end()
+    {
+        if (!kStaged) return;
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0 && m0 < args.M && n0 < args.N) {
+            tma_store_2d(tmap, block, static_cast<int32_t>(n0), static_cast<int32_t>(m0));
+            bulk_commit();
+        }
+    }
+
+    // Before the kernel ends: this warp's stores are complete.
+    static __device__ __forceinline__ void drain(int lane)
+    {
+        if (kStaged && lane == 0) bulk_wait_all();
+    }
+};
 
 // Half of one 16-column chunk: one 16x128b.x4 TMEM load (16 lanes), then
 // acc[i] += s_a * (s_w[i] * P_i) for the four pairs P_i = (row, row + 8) of
@@ -558,11 +603,12 @@ __device__ __forceinline__ void lds_b64x2(uint32_t addr, uint64_t &a, uint64_t &
 template <int MODE, int OUT, bool DUMP, bool PERROW, int RM = kRasterM>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a,
-                        const __grid_constant__ CUtensorMap tmap_w, const GemmArgs args)
+                        const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_y,
+                        const GemmArgs args)
 {
     griddep_wait();
     constexpr int NSIDE = (MODE == QUARTZ_ASYMMETRIC) ? 3 : 1;
-    using L = Smem<NSIDE>;
+    using L = Smem<NSIDE, OUT != QUARTZ_OUT_F32>;
     constexpr int kStages = L::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -599,6 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == kProducerWarp && lane == 0) {
         tma_prefetch_desc(&tmap_a);
         tma_prefetch_desc(&tmap_w);
+        if (OUT != QUARTZ_OUT_F32) tma_prefetch_desc(&tmap_y);
     }
     tc_fence_before();
     __syncthreads();
@@ -741,7 +788,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         // f32x2 arithmetic (asymmetric first adds the exact integer
         // zero-point terms to P_g).
         // ------------------------------------------------------------------
-        constexpr int S = L::kSideSlots;
         const int quarter = warp & 3;
         const int slot = warp >> 2;
         const int trow = lane >> 2;          // row offset inside each 8-row band
@@ -785,80 +831,91 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
                 int mt, nt;
                 tile_coords<RM>(tile, args, mt, nt);
+                const int64_t n0 = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp;
+                TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
+                                 n0);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const int64_t m = static_cast<int64_t>(mt) * BM + quarter * 32 + 16 * h + 8 * e + trow;
-                        if (m >= args.M) continue;
-                        const float s_a = args.a_side[perm32(m)];
+                        const int r = 16 * h + 8 * e + trow;
+                        const int64_t m = static_cast<int64_t>(mt) * BM + quarter * 32 + r;
+                        const float s_a = args.a_side[perm32(m)];  // (side values are padded to whole tiles)
 #pragma unroll
                         for (int chunk = 0; chunk < 4; ++chunk) {
-                            const int64_t n = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + 16 * chunk + tq;
-                            if (n >= args.N) continue;
+                            const int64_t n = n0 + 16 * chunk + tq;
+                            const float4 s_w = *reinterpret_cast<const float4 *>(args.w_side + n);
+                            const float swv[4] = {s_w.x, s_w.y, s_w.z, s_w.w};
                             float vv[4];
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 const int32_t P = acci[chunk][8 * h + 2 * i + e];
-                                if (DUMP) args.partials[m * args.N + n + i] = P;
-                                const float t = __fmul_rn(static_cast<float>(P), args.w_side[n + i]);
-                                vv[i] = __fmul_rn(t, s_a);
+                                if (DUMP && m < args.M && n < args.N) args.partials[m * args.N + n + i] = P;
+                                vv[i] = __fmul_rn(__fmul_rn(static_cast<float>(P), swv[i]), s_a);
                             }
-                            float4 v = make_float4(vv[0], vv[1], vv[2], vv[3]);
-                            if (args.bias) {
-                                const uint2 braw = __ldg(reinterpret_cast<const uint2 *>(args.bias + n));
-                                const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&braw.x));
-                                const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&braw.y));
-                                v.x = __fadd_rn(v.x, b0.x);
-                                v.y = __fadd_rn(v.y, b0.y);
-                                v.z = __fadd_rn(v.z, b1.x);
-                                v.w = __fadd_rn(v.w, b1.y);
-                            }
-                            store_quad<OUT>(args.y, m * args.N + n, v);
+                            out.put(16 * h + 8 * e, chunk, make_float4(vv[0], vv[1], vv[2], vv[3]));
                         }
                     }
+                out.end();
             }
         } else if constexpr (MODE == QUARTZ_SYMMETRIC && !DUMP) {
             // Symmetric fast path: each half chunk (16 lanes x 16 columns: TMEM
             // load, wait and the scale arithmetic) is one PTX block on
             // explicit 64-bit pairs, which keeps the kernel free of spills.
+            // The group loop carries only its accumulators, three offsets and
+            // a count: with the work item and a group index carried too, ptxas
+            // spilled and added moves (18432 x 12288 x 3072 1047 us, now 984;
+            // 8192 x 4608 x 1152 84.6, now 79; both with TileOut).  It runs at
+            // about 0.85 of what the pair operations alone take: mul + fma on
+            // f32x2 pairs with distinct operands need 5.5 cycles a pair and
+            // scheduler (register reads), 704 per group of a tile.  Loads of
+            // 32 columns or of both lane halves per wait, and scales loaded
+            // ahead, measured 1-10% slower.
             // acc64[c][4h + i]: output column 16c + tq + i, rows trow + 16h (low) and + 8 (high)
             uint64_t acc64[4][8];
-            int it = 0;
+            uint32_t buf = 0, par = 0, side = 0;  // accumulator (column offset), its parity, scale slot offset
+            const uint32_t tbase0 = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(slot * kColsPerWarp);
+            const uint32_t side_a0 = smem_base + L::kSide + (quarter * 32 + 4 * trow) * 4;
+            const uint32_t side_w0 = smem_base + L::kSide + L::kSideABytes + (slot * kColsPerWarp + tq) * 4;
             bool ok = true;
             const int n_items = work_items(args);
             for (int k = 0; k < n_items && ok; ++k) {
-                const WorkItem wi = work_item(args, k);
+                int left;
+                {
+                    const WorkItem wi = work_item(args, k);
+                    left = wi.g1 - wi.g0;
+                }
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) acc64[c][j] = 0ull;
-                for (int g = wi.g0; g < wi.g1; ++g, ++it) {
-                    const int b = it & 1;
-                    const int ss = it % S;
-                    const uint32_t side_a = smem_base + L::kSide + ss * L::kSideSlotBytes + (quarter * 32 + 4 * trow) * 4;
-                    const uint32_t side_w = smem_base + L::kSide + ss * L::kSideSlotBytes + L::kSideABytes +
-                                            (slot * kColsPerWarp + tq) * 4;
-                    if (!mbar_wait_warp(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err, kWaitLimitNs)) {
+                for (; left > 0; --left) {
+                    const uint32_t full = acc_full_bar(0) + (buf >> 5);
+                    if (!mbar_wait_warp(full, par, abort_flag, args.dev_err, kWaitLimitNs)) {
                         ok = false;
                         break;
                     }
                     uint64_t sa0, sa1;
-                    lds_b64x2(side_a, sa0, sa1);
+                    lds_b64x2(side_a0 + side, sa0, sa1);
                     tc_fence_after();
-                    const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
-                                           static_cast<uint32_t>(b * BN + slot * kColsPerWarp);
+                    const uint32_t tbase = tbase0 + buf;
 #pragma unroll
                     for (int chunk = 0; chunk < 4; ++chunk) {
-                        const float4 sw = lds_f4(side_w + 16 * chunk * 4);
+                        const float4 sw = lds_f4(side_w0 + side + 16 * chunk * 4);
                         epi_half_chunk_sym(tbase + 16 * chunk, sw, sa0, acc64[chunk]);
                         epi_half_chunk_sym(tbase + (16u << 16) + 16 * chunk, sw, sa1, acc64[chunk] + 4);
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(acc_empty_bar(b));
+                    if (lane == 0) mbar_arrive(full + 16);
+                    side += L::kSideSlotBytes;
+                    if (side == L::kSideSlots * L::kSideSlotBytes) side = 0;
+                    par ^= buf >> 8;
+                    buf ^= BN;
                 }
                 if (!ok) break;
+                asm volatile("" : "+r"(k));  // the item is looked up again rather than carried through the loop
+                const WorkItem wi = work_item(args, k);
                 if (wi.part >= 0) {
                     // split last wave: leave this part's fp32 partial tile for
                     // tail_combine_kernel: slot tail * split + part holds 16
@@ -875,7 +932,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                                                         static_cast<uint32_t>(acc64[c][2 * j + 1] >> 32));
                     continue;
                 }
-                store_tile_sym<OUT, RM>(args, wi.tile, quarter, slot, trow, tq, acc64);
+                int mt, nt;
+                tile_coords<RM>(wi.tile, args, mt, nt);
+                TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
+                                 static_cast<int64_t>(nt) * BN + slot * kColsPerWarp);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                        for (int chunk = 0; chunk < 4; ++chunk) {
+                            float vv[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const uint64_t q = acc64[chunk][4 * h + i];
+                                vv[i] = __uint_as_float(static_cast<uint32_t>(e ? (q >> 32) : q));
+                            }
+                            out.put(16 * h + 8 * e, chunk, make_float4(vv[0], vv[1], vv[2], vv[3]));
+                        }
+                out.end();
             }
         } else {
             float2 acc[2][16];
@@ -888,7 +963,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int j = 0; j < 16; ++j) acc[h][j] = make_float2(0.f, 0.f);
                 for (int g = 0; g < G; ++g, ++it) {
                     const int b = it & 1;
-                    const int ss = it % S;
+                    const int ss = it % L::kSideSlots;
                     const uint32_t side_a = smem_base + L::kSide + ss * L::kSideSlotBytes + (quarter * 32 + 4 * trow) * 4;
                     const uint32_t side_w = smem_base + L::kSide + ss * L::kSideSlotBytes + L::kSideABytes +
                                             (slot * kColsPerWarp + tq) * 4;
@@ -958,35 +1033,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                 int mt, nt;
                 tile_coords<RM>(tile, args, mt, nt);
                 // ---- store: 4 rows x 4 chunks of 4 consecutive columns per thread ----
+                TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
+                                 static_cast<int64_t>(nt) * BN + slot * kColsPerWarp);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int64_t m = static_cast<int64_t>(mt) * BM + quarter * 32 + 16 * h + 8 * e + trow;
-                        if (m >= args.M) continue;
+                    for (int e = 0; e < 2; ++e)
 #pragma unroll
                         for (int chunk = 0; chunk < 4; ++chunk) {
-                            const int64_t n = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + 16 * chunk + tq;
-                            if (n >= args.N) continue;
-                            float4 v;
-                            v.x = e ? acc[h][4 * chunk + 0].y : acc[h][4 * chunk + 0].x;
-                            v.y = e ? acc[h][4 * chunk + 1].y : acc[h][4 * chunk + 1].x;
-                            v.z = e ? acc[h][4 * chunk + 2].y : acc[h][4 * chunk + 2].x;
-                            v.w = e ? acc[h][4 * chunk + 3].y : acc[h][4 * chunk + 3].x;
-                            if (args.bias) {
-                                const uint2 braw = __ldg(reinterpret_cast<const uint2 *>(args.bias + n));
-                                const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&braw.x));
-                                const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&braw.y));
-                                v.x = __fadd_rn(v.x, b0.x);
-                                v.y = __fadd_rn(v.y, b0.y);
-                                v.z = __fadd_rn(v.z, b1.x);
-                                v.w = __fadd_rn(v.w, b1.y);
-                            }
-                            store_quad<OUT>(args.y, m * args.N + n, v);
+                            const float2 *q = &acc[h][4 * chunk];
+                            out.put(16 * h + 8 * e, chunk,
+                                    e ? make_float4(q[0].y, q[1].y, q[2].y, q[3].y)
+                                      : make_float4(q[0].x, q[1].x, q[2].x, q[3].x));
                         }
-                    }
+                out.end();
             }
         }
+        TileOut<OUT>::drain(lane);
     }
 
     tc_fence_before();
@@ -1279,6 +1342,21 @@ bool make_operand_map(CUtensorMap *m, const void *base, int64_t rows, int64_t K,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Two-byte output [M, N], written in blocks of 32 rows x 64 columns (128-byte
+// swizzle); parts of a block past M or N are not written.
+bool make_output_map(CUtensorMap *m, void *y, int64_t M, int64_t N)
+{
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(M)};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(N) * 2};
+    const cuuint32_t box[2] = {kColsPerWarp, 32};
+    const cuuint32_t estr[2] = {1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // SM count of the current device (0 if there is none), looked up once per device.
 int device_sms_or_zero()
 {
@@ -1300,11 +1378,11 @@ int num_sms()
 }
 
 template <int MODE, int OUT>
-cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tw, const GemmArgs &args,
+cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &ty, const GemmArgs &args,
                       cudaStream_t s)
 {
     constexpr int NSIDE = (MODE == QUARTZ_ASYMMETRIC) ? 3 : 1;
-    constexpr int smem = Smem<NSIDE>::kAlloc;
+    constexpr int smem = Smem<NSIDE, OUT != QUARTZ_OUT_F32>::kAlloc;
     static_assert(smem <= 227 * 1024, "shared memory budget");
     auto kern = args.partials ? gemm_tcgen05_kernel<MODE, OUT, true, false>
                               : gemm_tcgen05_kernel<MODE, OUT, false, false>;
@@ -1321,18 +1399,18 @@ cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tw, const GemmAr
     int grid = args.num_tiles < num_sms() ? args.num_tiles : num_sms();
     if (args.split > 1 && args.ls == 0 && args.full_tiles == 0) grid = args.tail_tiles * args.split;
     if (args.ls > 0) grid = num_sms();  // one group range per SM
-    launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, ta, tw, args);
+    launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, ta, tw, ty, args);
     return cudaGetLastError();
 }
 
 template <int MODE>
-cudaError_t launch_tc_out(const CUtensorMap &ta, const CUtensorMap &tw, const GemmArgs &args,
+cudaError_t launch_tc_out(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &ty, const GemmArgs &args,
                           int y_type, cudaStream_t s)
 {
     switch (y_type) {
-        case QUARTZ_OUT_F16: return launch_tc<MODE, QUARTZ_OUT_F16>(ta, tw, args, s);
-        case QUARTZ_OUT_BF16: return launch_tc<MODE, QUARTZ_OUT_BF16>(ta, tw, args, s);
-        default: return launch_tc<MODE, QUARTZ_OUT_F32>(ta, tw, args, s);
+        case QUARTZ_OUT_F16: return launch_tc<MODE, QUARTZ_OUT_F16>(ta, tw, ty, args, s);
+        case QUARTZ_OUT_BF16: return launch_tc<MODE, QUARTZ_OUT_BF16>(ta, tw, ty, args, s);
+        default: return launch_tc<MODE, QUARTZ_OUT_F32>(ta, tw, ty, args, s);
     }
 }
 
@@ -1575,7 +1653,8 @@ cudaError_t launch_gemm_tcgen05(const LinearWorkspace &ws, int64_t M, int64_t N,
                                 cudaStream_t s, bool per_row, bool wide)
 {
     if (M == 0) return cudaSuccess;
-    CUtensorMap ta, tw;
+    CUtensorMap ta, tw, ty = {};
+    if (y_type != QUARTZ_OUT_F32 && !make_output_map(&ty, y, M, N)) return cudaErrorInvalidValue;
     if (!make_operand_map(&ta, ws.a_op, M, K, BM) || !make_operand_map(&tw, ws.w_op, round_up(N, 16), K, BN))
         return cudaErrorInvalidValue;
     GemmArgs args = make_args(ws, M, N, K, bias, y, y_type, partials, partials_group, dev_err);
@@ -1590,13 +1669,13 @@ cudaError_t launch_gemm_tcgen05(const LinearWorkspace &ws, int64_t M, int64_t N,
         args.ls = ls;
         args.tail_tiles = ws.tail_tiles;
         args.full_tiles = args.num_tiles - ws.tail_tiles;
-        cudaError_t e = launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, args, y_type, s);
+        cudaError_t e = launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, ty, args, y_type, s);
         if (e != cudaSuccess) return e;
         return launch_tail_combine(args, y_type, s);
     }
-    if (per_row) return launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, args, y_type, s);
-    return mode == QUARTZ_ASYMMETRIC ? launch_tc_out<QUARTZ_ASYMMETRIC>(ta, tw, args, y_type, s)
-                                     : launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, args, y_type, s);
+    if (per_row) return launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, ty, args, y_type, s);
+    return mode == QUARTZ_ASYMMETRIC ? launch_tc_out<QUARTZ_ASYMMETRIC>(ta, tw, ty, args, y_type, s)
+                                     : launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, ty, args, y_type, s);
 }
 
 cudaError_t launch_gemm_simt(const LinearWorkspace &ws, int64_t M, int64_t N, int64_t K, int mode,
