@@ -172,10 +172,10 @@ size_t quartz_linear_workspace_size(int64_t M, int64_t N, int64_t K, const quart
 
 /* Kernels one quartz_linear_ex call with these sizes, algorithm and
  * partials setting launches on the current device: operand preparation,
- * the GEMM and, when the symmetric group-64 tcgen05 GEMM (no partials)
- * splits its last wave of tiles along K, the kernel that adds the parts in
- * a fixed order and writes those tiles.  Returns 0 for invalid arguments
- * or M = 0 (no launch). */
+ * the GEMM and, when the symmetric tcgen05 GEMM (no partials; groups of 64
+ * or one scale per row) splits its last wave of tiles along K, the kernel
+ * that adds the parts in a fixed order and writes those tiles.  Returns 0
+ * for invalid arguments or M = 0 (no launch). */
 int32_t quartz_linear_launch_count(int64_t M, int64_t N, int64_t K, const quartz_params_t *p, int32_t algo,
                                    int32_t with_partials);
 

@@ -169,7 +169,7 @@ int32_t quartz_linear_launch_count(int64_t M, int64_t N, int64_t K, const quartz
     if (algo != QUARTZ_ALGO_TCGEN05 && algo != QUARTZ_ALGO_SIMT && algo != QUARTZ_ALGO_SHIFT) return 0;
     if (M == 0) return 0;
     const bool split = algo == QUARTZ_ALGO_TCGEN05 && p->mode == QUARTZ_SYMMETRIC && !with_partials &&
-                       p->group_q == 64 && linear_tail_parts(M, N, K, p->mode) > 1;
+                       linear_tail_parts(M, N, K, p->mode, p->group_q != 64) > 1;
     return split ? 3 : 2;
 }
 

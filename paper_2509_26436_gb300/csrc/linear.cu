@@ -399,12 +399,6 @@ __device__ __forceinline__ WorkItem work_item(const GemmArgs &a, int k)
     return w;
 }
 
-// (a.x, a.y) += (b.x, b.y) on a packed fp32 pair.
-__device__ __forceinline__ void add2_rn(uint64_t &a, uint64_t b)
-{
-    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
-}
-
 // Two values rounded to a two-byte output type, the first in the low half.
 template <int OUT>
 __device__ __forceinline__ uint32_t pack2(float lo, float hi)
@@ -734,8 +728,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const WorkItem wi = work_item(args, k);
                 for (int g = wi.g0; g < wi.g1; ++g) {
                     const int b = ic & 1;
-                    const bool first = (g % CH) == 0;
-                    const bool last = (g % CH) == CH - 1 || g == G - 1;
+                    const bool first = ((g - wi.g0) % CH) == 0;
+                    const bool last = ((g - wi.g0) % CH) == CH - 1 || g == wi.g1 - 1;
                     if (!mbar_wait_warp(full_bar(s), phase, abort_flag, args.dev_err, kWaitLimitNs) ||
                         (first && ic >= 2 && !mbar_wait_warp(acc_empty_bar(b), ((ic >> 1) - 1) & 1, abort_flag,
                                                              args.dev_err, kWaitLimitNs))) {
@@ -804,8 +798,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             int32_t acci[4][16];
             int ic = 0;
             bool ok = true;
-            const int nchunks = (G + kPerRowChunk - 1) / kPerRowChunk;
-            for (int tile = blockIdx.x; tile < args.num_tiles && ok; tile += gridDim.x) {
+            const int n_items = work_items(args);
+            for (int k = 0; k < n_items && ok; ++k) {
+                const WorkItem wi = work_item(args, k);
+                const int nchunks = (wi.g1 - wi.g0 + kPerRowChunk - 1) / kPerRowChunk;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -829,8 +825,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 0) mbar_arrive(acc_empty_bar(b));
                 }
                 if (!ok) break;
+                if (!DUMP && wi.part >= 0) {  // a cut tile: this part's integer sums (planes as below)
+                    uint4 *dst = reinterpret_cast<uint4 *>(args.tail_part) +
+                                 ((wi.tail * args.split + wi.part) * 16 * (kEpiWarps * 32) + warp * 32 + lane);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            dst[(4 * c + j) * (kEpiWarps * 32)] =
+                                make_uint4(static_cast<uint32_t>(acci[c][4 * j]), static_cast<uint32_t>(acci[c][4 * j + 1]),
+                                           static_cast<uint32_t>(acci[c][4 * j + 2]), static_cast<uint32_t>(acci[c][4 * j + 3]));
+                    continue;
+                }
                 int mt, nt;
-                tile_coords<RM>(tile, args, mt, nt);
+                tile_coords<RM>(wi.tile, args, mt, nt);
                 const int64_t n0 = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp;
                 TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
                                  n0);
@@ -1064,7 +1072,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // partial tiles in part order, then stores the sum as the epilogue would
 // have.  Grid: (tail tile, 16-column chunk c of every warp's slice); block:
 // one thread per epilogue thread, which owns the chunk's 8 column pairs.
-template <int OUT>
+template <int OUT, bool PERROW>
 __global__ void __launch_bounds__(kEpiWarps * 32) tail_combine_kernel(const __grid_constant__ GemmArgs args)
 {
     griddep_wait();
@@ -1078,20 +1086,22 @@ __global__ void __launch_bounds__(kEpiWarps * 32) tail_combine_kernel(const __gr
     if (parts == 1) return;  // the tile lies in one CTA's range: stored whole by the GEMM
     const uint4 *src = reinterpret_cast<const uint4 *>(args.tail_part) +
                        static_cast<int64_t>(tail) * args.split * 16 * T + 4 * c * T + threadIdx.x;
-    uint64_t acc[8];
+    uint32_t acc[16];  // acc[4i' ..]: pairs (row, row + 8) of the chunk's columns, as the epilogue holds them
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const uint4 v = __ldcg(src + j * T);
-        acc[2 * j] = (static_cast<uint64_t>(v.y) << 32) | v.x;
-        acc[2 * j + 1] = (static_cast<uint64_t>(v.w) << 32) | v.z;
+        acc[4 * j] = v.x, acc[4 * j + 1] = v.y, acc[4 * j + 2] = v.z, acc[4 * j + 3] = v.w;
     }
     for (int p = 1; p < parts; ++p) {
         const uint4 *sp = src + static_cast<int64_t>(p) * 16 * T;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const uint4 v = __ldcg(sp + j * T);
-            add2_rn(acc[2 * j], (static_cast<uint64_t>(v.y) << 32) | v.x);
-            add2_rn(acc[2 * j + 1], (static_cast<uint64_t>(v.w) << 32) | v.z);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                acc[4 * j + i] = PERROW ? acc[4 * j + i] + w[i]
+                                        : __float_as_uint(__fadd_rn(__uint_as_float(acc[4 * j + i]), __uint_as_float(w[i])));
         }
     }
     int mt, nt;
@@ -1110,8 +1120,12 @@ __global__ void __launch_bounds__(kEpiWarps * 32) tail_combine_kernel(const __gr
             if (m >= args.M) continue;
             float vv[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                vv[i] = __uint_as_float(static_cast<uint32_t>(e ? (acc[4 * h + i] >> 32) : acc[4 * h + i]));
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t q = acc[8 * h + 2 * i + e];
+                vv[i] = PERROW ? __fmul_rn(__fmul_rn(static_cast<float>(static_cast<int32_t>(q)), args.w_side[n + i]),
+                                           args.a_side[perm32(m)])
+                               : __uint_as_float(q);
+            }
             store_quad<OUT>(args.y, m * args.N + n, add_bias4(args, n, make_float4(vv[0], vv[1], vv[2], vv[3])));
         }
 }
@@ -1414,13 +1428,14 @@ cudaError_t launch_tc_out(const CUtensorMap &ta, const CUtensorMap &tw, const CU
     }
 }
 
+template <bool PERROW>
 cudaError_t launch_tail_combine(const GemmArgs &args, int y_type, cudaStream_t s)
 {
     const unsigned grid = static_cast<unsigned>(args.tail_tiles) * 4;
     switch (y_type) {
-        case QUARTZ_OUT_F16: launch_pdl(tail_combine_kernel<QUARTZ_OUT_F16>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
-        case QUARTZ_OUT_BF16: launch_pdl(tail_combine_kernel<QUARTZ_OUT_BF16>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
-        default: launch_pdl(tail_combine_kernel<QUARTZ_OUT_F32>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
+        case QUARTZ_OUT_F16: launch_pdl(tail_combine_kernel<QUARTZ_OUT_F16, PERROW>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
+        case QUARTZ_OUT_BF16: launch_pdl(tail_combine_kernel<QUARTZ_OUT_BF16, PERROW>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
+        default: launch_pdl(tail_combine_kernel<QUARTZ_OUT_F32, PERROW>, dim3(grid), dim3(kEpiWarps * 32), 0, s, args); break;
     }
     return cudaGetLastError();
 }
@@ -1540,10 +1555,33 @@ void tail_split(int64_t M, int64_t N, int64_t K, int mode, int *tail, int *split
     *split = static_cast<int>(S);
 }
 
-int linear_tail_parts(int64_t M, int64_t N, int64_t K, int mode)
+// With scales per row the same plan cuts the int32 sums (exact, so the cut
+// changes no result).  A 64-wide stage takes about 0.27 us there, so it is
+// taken only where the busiest CTA is spared kMinRowSaving of them, or
+// kMinRowRangeSaving in the range forms, which leave more partial tiles.  GEMM
+// + combine against whole tiles: 2048 x 1280 x 11520 (ranges, spares 85) 51.9
+// -> 41.6 us, 2048 x 1280 x 5760 (42) 31.4 -> 31.4, 2560 x 3072 x 5120 (two
+// waves, 34) 49.8 -> 53.9; 8192 x 640 x 5760 (3 parts, 60) 53.9 -> 45.7, 1790 x
+// 3064 x 3072 (36) 35.5 -> 31.4, 1000 x 1304 x 2048 (21) 17.1 -> 17.0, 1000 x
+// 1304 x 1152 (12) 15.0 -> 17.0.
+constexpr int kMinRowSaving = 32;
+constexpr int kMinRowRangeSaving = 48;
+
+bool row_split_pays(int64_t M, int64_t N, int64_t K, int tail, int split, int ls)
 {
-    int tail = 0, split = 1;
-    tail_split(M, N, K, mode, &tail, &split);
+    const int sms = num_sms();
+    const int64_t T = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), G = K / kGroupQ;
+    const int64_t P = T < sms ? T : sms;
+    const int64_t whole = (T + P - 1) / P * G;
+    const int64_t cut = (T - tail) / P * G + (ls > 0 ? ls : (G + split - 1) / split);
+    return whole - cut >= (ls > 0 ? kMinRowRangeSaving : kMinRowSaving);
+}
+
+int linear_tail_parts(int64_t M, int64_t N, int64_t K, int mode, bool per_row)
+{
+    int tail = 0, split = 1, ls = 0;
+    tail_split(M, N, K, mode, &tail, &split, &ls);
+    if (per_row && split > 1 && !row_split_pays(M, N, K, tail, split, ls)) return 1;
     return split;
 }
 
@@ -1662,8 +1700,9 @@ cudaError_t launch_gemm_tcgen05(const LinearWorkspace &ws, int64_t M, int64_t N,
     args.wide = wide ? 1 : 0;
     if (mode == QUARTZ_SYMMETRIC && !partials && !per_row && args.tiles_n <= kRowRasterMaxN) args.raster_m = 1;
     int tail = 0, split = 1, ls = 0;  // the workspace's split must still match this device's grid
-    if (mode == QUARTZ_SYMMETRIC && !partials && !per_row && ws.tail_split > 1 && ws.tail_part)
+    if (mode == QUARTZ_SYMMETRIC && !partials && ws.tail_split > 1 && ws.tail_part)
         tail_split(M, N, K, mode, &tail, &split, &ls);
+    if (per_row && split > 1 && !row_split_pays(M, N, K, tail, split, ls)) split = 1;
     if (split > 1 && split == ws.tail_split && tail == ws.tail_tiles && ls == ws.tail_ls) {
         args.split = ws.tail_split;
         args.ls = ls;
@@ -1671,7 +1710,7 @@ cudaError_t launch_gemm_tcgen05(const LinearWorkspace &ws, int64_t M, int64_t N,
         args.full_tiles = args.num_tiles - ws.tail_tiles;
         cudaError_t e = launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, ty, args, y_type, s);
         if (e != cudaSuccess) return e;
-        return launch_tail_combine(args, y_type, s);
+        return per_row ? launch_tail_combine<true>(args, y_type, s) : launch_tail_combine<false>(args, y_type, s);
     }
     if (per_row) return launch_tc_out<QUARTZ_SYMMETRIC>(ta, tw, ty, args, y_type, s);
     return mode == QUARTZ_ASYMMETRIC ? launch_tc_out<QUARTZ_ASYMMETRIC>(ta, tw, ty, args, y_type, s)

@@ -91,7 +91,7 @@ struct LinearWorkspace {
 size_t linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int mode);
 // Parts each tile of the symmetric tcgen05 GEMM's split last wave is cut
 // into on the current device (1: no split).
-int linear_tail_parts(int64_t M, int64_t N, int64_t K, int mode);
+int linear_tail_parts(int64_t M, int64_t N, int64_t K, int mode, bool per_row);
 void linear_workspace_carve(void *base, int64_t M, int64_t N, int64_t K, int mode,
                             LinearWorkspace *ws);
 // Expands the operands to E4M3 and transposes their scales into the
