@@ -16,6 +16,7 @@ from __future__ import annotations
 
 import ctypes as C
 from dataclasses import dataclass
+from functools import lru_cache
 
 from . import _native as N
 from ._native import (ALGO_SHIFT, ALGO_SIMT, ALGO_TCGEN05, ASYMMETRIC, OUT_BF16, OUT_F16, OUT_F32,  # noqa: F401
@@ -27,9 +28,17 @@ __all__ = ["Params", "Encoded", "quantize", "encode_weights", "dequantize", "lin
            "SYMMETRIC", "ASYMMETRIC", "QuartzError"]
 
 
+_byref = C.byref
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    """torch, imported on the first use of a tensor."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 @dataclass(frozen=True)
@@ -49,6 +58,12 @@ class Params:
         return N.QuartzParams(self.group_q, self.group_s, self.mode, self.flag_bits, self.code_bits)
 
 
+@lru_cache(maxsize=256)
+def _c_params(params: Params) -> N.QuartzParams:
+    """The C struct of `params` (plain numbers; only ever read)."""
+    return params.c()
+
+
 class Encoded:
     """An encoded [rows, K] tensor on the GPU (Section 4.4 storage format):
     codes uint8 [rows, K/2], flags uint8 [rows, K/G_s], scales fp16
@@ -60,9 +75,11 @@ class Encoded:
         self.rows, self.K, self.params = rows, K, params
 
     def c(self) -> N.QuartzEncoded:
-        ptr = lambda t: None if t is None else t.data_ptr()  # noqa: E731
-        return N.QuartzEncoded(ptr(self.codes), ptr(self.flags), ptr(self.scales), ptr(self.zeros),
-                               ptr(self.gsum), self.rows, self.K, self.params.c())
+        codes, flags, scales, zeros, gsum = self.codes, self.flags, self.scales, self.zeros, self.gsum
+        return N.QuartzEncoded(None if codes is None else codes.data_ptr(), None if flags is None else flags.data_ptr(),
+                               None if scales is None else scales.data_ptr(),
+                               None if zeros is None else zeros.data_ptr(), None if gsum is None else gsum.data_ptr(),
+                               self.rows, self.K, _c_params(self.params))
 
     @property
     def nbytes(self) -> int:
@@ -70,11 +87,13 @@ class Encoded:
         return sum(t.numel() * t.element_size() for t in ts if t is not None)
 
 
+_Sizes = C.c_size_t * 5
+
+
 def empty_encoded(rows: int, K: int, params: Params = Params(), device="cuda") -> Encoded:
     torch = _torch()
-    sizes = (C.c_size_t * 5)()
-    p = params.c()
-    N.check(N.load().quartz_encoded_sizes(rows, K, C.byref(p), sizes), "quartz_encoded_sizes")
+    sizes = _Sizes()
+    N.check(N.load().quartz_encoded_sizes(rows, K, _byref(_c_params(params)), sizes), "quartz_encoded_sizes")
     G = K // params.group_q
     codes = torch.empty((rows, K // 2), dtype=torch.uint8, device=device)
     if params.flag_bits == 4:
@@ -89,15 +108,30 @@ def empty_encoded(rows: int, K: int, params: Params = Params(), device="cuda") -
     return Encoded(codes, flags, scales, zeros, gsum, rows, K, params)
 
 
+_raw_stream = None  # (device getter, stream getter) once CUDA is initialised
+
+
 def _stream(stream=None) -> int:
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    """The cudaStream_t of `stream`, or of the current stream of the current
+    device (read through the raw accessors where torch has them: 0.2 us
+    against 3 us for building a Stream object, of a call of about 15)."""
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        torch = _torch()
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if not torch.cuda.is_initialized() or device is None or raw is None:
+            return torch.cuda.current_stream().cuda_stream
+        _raw_stream = (device, raw)
+    device, raw = _raw_stream
+    return raw(device())
 
 
 def _check_f16(x, name):
     torch = _torch()
-    if not (x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.is_contiguous()):
+    if not (x.is_cuda and x.dtype is torch.float16 and x.dim() == 2 and x.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous 2-D float16 CUDA tensor")
 
 
@@ -111,7 +145,7 @@ def quantize(x, group_s: int = 16, mode: int = SYMMETRIC, out: Encoded | None = 
     e = out if out is not None else empty_encoded(rows, K, Params(group_q, group_s, mode, flag_bits, code_bits),
                                                   x.device)
     ec = e.c()
-    N.check(getattr(N.load(), _entry)(x.data_ptr(), C.byref(ec), _stream(stream)), _entry)
+    N.check(getattr(N.load(), _entry)(x.data_ptr(), _byref(ec), _stream(stream)), _entry)
     return e
 
 
@@ -133,7 +167,7 @@ def quantize_static(x, scale, group_s: int = 16, group_q: int = 64, out: Encoded
     e = out if out is not None else empty_encoded(rows, K, Params(group_q, group_s, SYMMETRIC, flag_bits), x.device)
     ec = e.c()
     bits = int(np.float16(scale).view(np.uint16))
-    N.check(N.load().quartz_quantize_static(x.data_ptr(), bits, C.byref(ec), _stream(stream)),
+    N.check(N.load().quartz_quantize_static(x.data_ptr(), bits, _byref(ec), _stream(stream)),
             "quartz_quantize_static")
     return e
 
@@ -145,37 +179,39 @@ def dequantize(e: Encoded, stream=None, out=None):
     if not (y.is_cuda and y.dtype == torch.float16 and y.is_contiguous() and y.numel() == e.rows * e.K):
         raise ValueError("out must be a contiguous float16 CUDA tensor of rows x K elements")
     ec = e.c()
-    N.check(N.load().quartz_dequantize(C.byref(ec), y.data_ptr(), _stream(stream)), "quartz_dequantize")
+    N.check(N.load().quartz_dequantize(_byref(ec), y.data_ptr(), _stream(stream)), "quartz_dequantize")
     return y
 
 
 def linear_workspace_size(M: int, N_: int, K: int, params: Params = Params()) -> int:
-    p = params.c()
-    return int(N.load().quartz_linear_workspace_size(M, N_, K, C.byref(p)))
+    return N.load().quartz_linear_workspace_size(M, N_, K, _byref(_c_params(params)))
 
 
 def linear_launch_count(M: int, N_: int, K: int, params: Params = Params(), algo: int = ALGO_TCGEN05,
                         partials: bool = False) -> int:
     """Kernels one linear() call with these sizes launches on the current
     device (0: invalid arguments or M = 0)."""
-    p = params.c()
-    return int(N.load().quartz_linear_launch_count(M, N_, K, C.byref(p), algo, 1 if partials else 0))
+    return N.load().quartz_linear_launch_count(M, N_, K, _byref(_c_params(params)), algo, 1 if partials else 0)
 
 
 _OUT = {"float16": OUT_F16, "bfloat16": OUT_BF16, "float32": OUT_F32}
+
+
+@lru_cache(maxsize=None)
+def _out_type(dtype) -> int:
+    return _OUT[str(dtype).replace("torch.", "")]
 
 
 def prepare_weights(w: Encoded, stream=None):
     """The weights' tensor-core operand and scale side values, prepared once
     (offline, like the encoding) for linear(..., w_prepared=...)."""
     torch = _torch()
-    p = w.params.c()
-    n = int(N.load().quartz_prepared_weights_size(w.rows, w.K, C.byref(p)))
+    n = N.load().quartz_prepared_weights_size(w.rows, w.K, _byref(_c_params(w.params)))
     if n == 0:
         raise ValueError("invalid weight shape for preparation")
     buf = torch.empty(n, dtype=torch.uint8, device=w.codes.device)
     wc = w.c()
-    N.check(N.load().quartz_prepare_weights(C.byref(wc), buf.data_ptr(), n, _stream(stream)),
+    N.check(N.load().quartz_prepare_weights(_byref(wc), buf.data_ptr(), n, _stream(stream)),
             "quartz_prepare_weights")
     return buf
 
@@ -196,7 +232,7 @@ def linear(a: Encoded, w: Encoded, bias=None, out_dtype=None, out=None, workspac
     M, Nn = a.rows, w.rows
     dev = a.codes.device
     y = out if out is not None else torch.empty((M, Nn), dtype=out_dtype, device=dev)
-    y_type = _OUT[str(y.dtype).replace("torch.", "")]
+    y_type = _out_type(y.dtype)
     if workspace is None:
         workspace = torch.empty(max(linear_workspace_size(M, Nn, a.K, a.params), 16),
                                 dtype=torch.uint8, device=dev)
@@ -219,8 +255,8 @@ def linear(a: Encoded, w: Encoded, bias=None, out_dtype=None, out=None, workspac
                               None if gemm_events is None else gemm_events[1].cuda_event,
                               None if w_prepared is None else w_prepared.data_ptr())
     rc = N.load().quartz_linear_ex(
-        C.byref(ac), C.byref(wc), None if bias is None else bias.data_ptr(), y.data_ptr(), y_type,
-        workspace.data_ptr(), workspace.numel() * workspace.element_size(), C.byref(opts),
+        _byref(ac), _byref(wc), None if bias is None else bias.data_ptr(), y.data_ptr(), y_type,
+        workspace.data_ptr(), workspace.numel() * workspace.element_size(), _byref(opts),
         _stream(stream))
     N.check(rc, "quartz_linear_ex")
     return y if part is None else (y, part)
@@ -239,7 +275,7 @@ def linear_f16(x, w: Encoded, bias=None, out_dtype=None, out=None, workspace=Non
     M, K = x.shape
     Nn = w.rows
     y = out if out is not None else torch.empty((M, Nn), dtype=out_dtype, device=x.device)
-    y_type = _OUT[str(y.dtype).replace("torch.", "")]
+    y_type = _out_type(y.dtype)
     if workspace is None:
         workspace = torch.empty(max(linear_workspace_size(M, Nn, K, w.params), 16),
                                 dtype=torch.uint8, device=x.device)
@@ -248,9 +284,9 @@ def linear_f16(x, w: Encoded, bias=None, out_dtype=None, out=None, workspace=Non
     wc = w.c()
     ac = a_out.c() if a_out is not None else None
     rc = N.load().quartz_linear_f16_ex(
-        x.data_ptr(), M, C.byref(wc), None if w_prepared is None else w_prepared.data_ptr(),
+        x.data_ptr(), M, _byref(wc), None if w_prepared is None else w_prepared.data_ptr(),
         None if bias is None else bias.data_ptr(), y.data_ptr(), y_type,
-        None if ac is None else C.byref(ac), workspace.data_ptr(),
+        None if ac is None else _byref(ac), workspace.data_ptr(),
         workspace.numel() * workspace.element_size(), _stream(stream))
     N.check(rc, "quartz_linear_f16_ex")
     return y
@@ -287,7 +323,7 @@ def probe_mma_f8(blocks: int, iters: int, stream=None) -> int:
 # --- attention decode step (Appendix D, Table 6) ----------------------------
 
 def attention_workspace_size(BH: int, L: int) -> int:
-    return int(N.load().quartz_attention_workspace_size(BH, L))
+    return N.load().quartz_attention_workspace_size(BH, L)
 
 
 def kv_append(x, cache: Encoded, L_max: int, t0: int, stream=None) -> None:
@@ -297,7 +333,7 @@ def kv_append(x, cache: Encoded, L_max: int, t0: int, stream=None) -> None:
         raise ValueError("x must be a contiguous [BH, T, d] float16 CUDA tensor")
     BH, T, _ = x.shape
     cc = cache.c()
-    N.check(N.load().quartz_kv_append(x.data_ptr(), BH, T, C.byref(cc), L_max, t0, _stream(stream)),
+    N.check(N.load().quartz_kv_append(x.data_ptr(), BH, T, _byref(cc), L_max, t0, _stream(stream)),
             "quartz_kv_append")
 
 
@@ -309,11 +345,11 @@ def attention_decode(q: Encoded, k_cache: Encoded, v_cache: Encoded, L_max: int,
     out_dtype = out_dtype or torch.float16
     dev = q.codes.device
     o = out if out is not None else torch.empty((q.rows, q.K), dtype=out_dtype, device=dev)
-    o_type = _OUT[str(o.dtype).replace("torch.", "")]
+    o_type = _out_type(o.dtype)
     if workspace is None:
         workspace = torch.empty(max(attention_workspace_size(q.rows, L), 16), dtype=torch.uint8, device=dev)
     qc, kc, vc = q.c(), k_cache.c(), v_cache.c()
-    N.check(N.load().quartz_attention_decode(C.byref(qc), C.byref(kc), C.byref(vc), L_max, L, float(scale),
+    N.check(N.load().quartz_attention_decode(_byref(qc), _byref(kc), _byref(vc), L_max, L, float(scale),
                                              o.data_ptr(), o_type, workspace.data_ptr(),
                                              workspace.numel() * workspace.element_size(), _stream(stream)),
             "quartz_attention_decode")

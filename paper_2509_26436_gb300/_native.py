@@ -92,6 +92,8 @@ _lib = None
 def load(path: str = LIB_PATH):
     """Load libquartz.so and declare every entry point; raises if missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(path):
