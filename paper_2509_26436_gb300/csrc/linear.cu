@@ -399,6 +399,12 @@ __device__ __forceinline__ WorkItem work_item(const GemmArgs &a, int k)
     return w;
 }
 
+// (a.x, a.y) += (b.x, b.y) on a packed fp32 pair.
+__device__ __forceinline__ void add2_rn(uint64_t &a, uint64_t b)
+{
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+}
+
 // Two values rounded to a two-byte output type, the first in the low half.
 template <int OUT>
 __device__ __forceinline__ uint32_t pack2(float lo, float hi)
@@ -472,17 +478,24 @@ struct TileOut {
     }
 
     // v: columns 16 chunk + tq .. + 3 of row r8 + trow (r8: 0, 8, 16, 24) of
-    // the slice; the bias is added in fp32, then one rounding to the output
-    // type.
-    __device__ __forceinline__ void put(int r8, int chunk, float4 v)
+    // the slice, rounded once to the output type.
+    __device__ __forceinline__ void put_raw(int r8, int chunk, float4 v)
     {
-        const int64_t m = m0 + r8 + trow, n = n0 + 16 * chunk + tq;
-        if (n < args.N) v = add_bias4(args, n, v);
         if (kStaged) {
             sts_b64(at + r8 * 128 + ((32u * chunk) ^ swz), pack2<OUT>(v.x, v.y), pack2<OUT>(v.z, v.w));
-        } else if (m < args.M && n < args.N) {
-            *reinterpret_cast<float4 *>(static_cast<float *>(args.y) + m * args.N + n) = v;
+        } else {
+            const int64_t m = m0 + r8 + trow, n = n0 + 16 * chunk + tq;
+            if (m < args.M && n < args.N)
+                *reinterpret_cast<float4 *>(static_cast<float *>(args.y) + m * args.N + n) = v;
         }
+    }
+
+    // The same after adding the bias in fp32.
+    __device__ __forceinline__ void put(int r8, int chunk, float4 v)
+    {
+        const int64_t n = n0 + 16 * chunk + tq;
+        if (n < args.N) v = add_bias4(args, n, v);
+        put_raw(r8, chunk, v);
     }
 
     __device__ __forceinline__ void end()
@@ -944,6 +957,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tile_coords<RM>(wi.tile, args, mt, nt);
                 TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
                                  static_cast<int64_t>(nt) * BN + slot * kColsPerWarp);
+                // (the bias goes into the accumulators, once per column, rather than
+                // through every put: 1-3% of a short tile)
+                if (args.bias) {
+#pragma unroll
+                    for (int chunk = 0; chunk < 4; ++chunk) {
+                        const int64_t n = out.n0 + 16 * chunk + tq;
+                        if (n < args.N) {
+                            const float4 b = add_bias4(args, n, make_float4(0.f, 0.f, 0.f, 0.f));
+                            const float bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                add2_rn(acc64[chunk][i], (static_cast<uint64_t>(__float_as_uint(bv[i & 3])) << 32) | __float_as_uint(bv[i & 3]));
+                        }
+                    }
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -956,7 +984,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 const uint64_t q = acc64[chunk][4 * h + i];
                                 vv[i] = __uint_as_float(static_cast<uint32_t>(e ? (q >> 32) : q));
                             }
-                            out.put(16 * h + 8 * e, chunk, make_float4(vv[0], vv[1], vv[2], vv[3]));
+                            out.put_raw(16 * h + 8 * e, chunk, make_float4(vv[0], vv[1], vv[2], vv[3]));
                         }
                 out.end();
             }
