@@ -65,12 +65,53 @@ __host__ __device__ __forceinline__ int64_t perm16(int64_t r)
 //   expand A, expand W: 16 codes per thread (8 bytes in, 16 E4M3 bytes out);
 //     the weight operand is row-permuted (perm16) and zero-padded to a
 //     multiple of 16 rows;
-//   side A, side W: side[0][g][.] = s[r, g]; asymmetric adds side[1] = z and
-//     side[2] = (is_a ? 64 z - gsum : gsum), so that the epilogue's integer
-//     correction is P + z_w * (64 z_a - A_g) - z_a * W_g.  Rows in
-//     [rows, rows_pad) are 0; weight rows are stored in natural order,
-//     activation rows at perm32(r).  One thread per row and 8 groups: its
-//     reads stay in L1 lines, consecutive threads write consecutive rows.
+//   side A, side W: side[0][g][.] = s[r, g], weight rows in natural order,
+//     activation rows at perm32(r); asymmetric adds a ZeroRec per row and
+//     group (see there) in the space of two more such planes.  Rows in
+//     [rows, rows_pad) are 0.  One thread per row and 8 groups: its reads stay
+//     in L1 lines, consecutive threads write consecutive rows.
+// Zero-point terms of one row and group.  With u = 64 z_a - A_g (A_g, W_g: the
+// gsum side values) the integer correction is P + z_w u - z_a W_g, the dot
+// product of an activation record (hi u, lo u, -z_a, -z_a) and a weight
+// record (z_w, z_w, hi W, lo W), hi x the multiple of 16 toward zero and lo x
+// the rest: |u| <= 64 * 128 + 64 * 112 < 2^14 and |W| <= 64 * 112, so every
+// entry is exact in fp16 and the tensor core adds the correction to P_g in
+// its fp32 accumulator, all integers below 2^23, as a K = 16 step of which 4
+// are used.  Against two more fused multiply-adds per output and group in the
+// epilogue (GEMM, CUDA events): 18432 x 3072 x 3072 461 -> 277 us, 4001 x 3456
+// x 1152 53.9 -> 37.5; results are the same bits.  Activation records are stored in row order, weight records in
+// operand order (perm16), the order of the GEMM's accumulator.
+struct ZeroRec {
+    __half v[4];
+};
+static_assert(sizeof(ZeroRec) == 8, "two 4-byte planes hold the records");
+
+__device__ __forceinline__ ZeroRec zero_rec(int z, int gsum, bool is_a)
+{
+    const int x = is_a ? kGroupQ * z - gsum : gsum;
+    const int lo = x % 16;
+    const __half hx = __int2half_rn(x - lo), lx = __int2half_rn(lo), hz = __int2half_rn(is_a ? -z : z);
+    ZeroRec r;
+    r.v[0] = is_a ? hx : hz;
+    r.v[1] = is_a ? lx : hz;
+    r.v[2] = is_a ? hz : hx;
+    r.v[3] = is_a ? hz : lx;
+    return r;
+}
+
+// (z_a, u) of an activation record, (z_w, W) of a weight record.
+__device__ __forceinline__ float2 zero_terms(const ZeroRec &r, bool is_a)
+{
+    const float a = __half2float(r.v[0]), b = __half2float(r.v[1]), c = __half2float(r.v[2]), d = __half2float(r.v[3]);
+    return is_a ? make_float2(-c, a + b) : make_float2(a, c + d);
+}
+
+// The records that follow the scale plane [G][rows_pad].
+__host__ __device__ __forceinline__ const ZeroRec *zero_recs(const float *side, int64_t G, int64_t rows_pad)
+{
+    return reinterpret_cast<const ZeroRec *>(side + G * rows_pad);
+}
+
 struct ExpandJob {
     const uint2 *codes;          // [rows, K/16] units of 16 codes
     const uint8_t *flags;        // [rows, K/G_s]
@@ -182,17 +223,15 @@ __device__ __forceinline__ void run_side(const SideJob &j, int64_t t, int G, int
     const int g0 = static_cast<int>(t / j.rows_pad) * kSideGroupsPerThread;
     if (g0 >= G) return;
     const int g1 = min(g0 + kSideGroupsPerThread, G);
-    const int64_t total = j.rows_pad * G;
-    const int64_t o = j.is_a ? perm32(r) : r;
+    ZeroRec *recs = const_cast<ZeroRec *>(zero_recs(j.side, G, j.rows_pad));
+    const int64_t o = j.is_a ? perm32(r) : r, oz = j.is_a ? r : perm16(r);
     const bool in = r < j.rows;
     for (int g = g0; g < g1; ++g) {
         const int64_t i = static_cast<int64_t>(g) * j.rows_pad + o;
         j.side[i] = in ? __half2float(j.scales[r * G + g]) : 0.f;
         if (nside > 1) {
-            const float z = in ? static_cast<float>(j.zeros[r * G + g]) : 0.f;
-            const float gs = in ? static_cast<float>(j.gsum[r * G + g]) : 0.f;
-            j.side[total + i] = z;
-            j.side[2 * total + i] = j.is_a ? (static_cast<float>(kGroupQ) * z - gs) : gs;
+            recs[static_cast<int64_t>(g) * j.rows_pad + oz] =
+                in ? zero_rec(j.zeros[r * G + g], j.gsum[r * G + g], j.is_a != 0) : zero_rec(0, 0, j.is_a != 0);
         }
     }
 }
@@ -221,7 +260,6 @@ constexpr int BN = 256;
 constexpr int BK = kGroupQ;
 constexpr int kABytes = BM * BK;      // E4M3 operands: one byte per element
 constexpr int kBBytes = BN * BK;
-constexpr int kStageBytes = kABytes + kBBytes;
 // Warpgroups 0-3 dequantise (16 warps: four per 32-lane TMEM quarter, 64
 // columns each); warpgroup 4 holds the TMA producer, the MMA issuer and two
 // idle warps.  The dequant epilogue is the throughput-critical part (two fp32
@@ -245,6 +283,8 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 4) * 32;
 constexpr int kProducerWarp = kEpiWarps;
 constexpr int kMmaWarp = kEpiWarps + 1;
+constexpr int kRecWarp = kEpiWarps + 2;  // zero-point records (asymmetric)
+constexpr int kRecDepth = 3;             // groups of record copies in flight (below the stage count)
 constexpr int kColsPerWarp = BN / 4;
 // Register split (setmaxnreg): 640 threads launch with 96 registers each;
 // warpgroup 4 drops to 32 so the epilogue warpgroups can hold 112
@@ -264,8 +304,8 @@ constexpr int kRowRasterMaxN = 16;  // see tile_coords
 constexpr int kPerRowChunk = 4;           // tiles are visited in bands of 8 M-tiles
 
 struct GemmArgs {
-    const float *a_side;  // [nside][G][m_pad]
-    const float *w_side;  // [nside][G][n_pad]
+    const float *a_side;  // scales [G][m_pad], then (asymmetric) the ZeroRecs [G][m_pad]
+    const float *w_side;  // scales [G][n_pad], then (asymmetric) the ZeroRecs [G][n_pad]
     int64_t m_pad, n_pad;
     int M, N, G;
     int tiles_m, tiles_n, num_tiles;
@@ -295,26 +335,36 @@ struct GemmArgs {
 };
 
 // Shared memory: the operand stages, the output blocks (one per epilogue warp,
-// see TileOut), then a ring of side-value slots (one group's NSIDE x BM
-// activation and NSIDE x BN weight values each), then the mbarriers.  5
-// stages cover the copy latency (a group takes 350 cycles or more; 4, 6 and 8
-// measured no better).  A group's side values are copied with its operands and counted
-// on the same barrier.  A slot needs no barrier of its own to be reused: the
+// see TileOut), then a ring of scale slots (one group's BM activation and BN
+// weight scales each), then the mbarriers.  5 stages (4 with zero points)
+// cover the copy latency (a group takes 350 cycles or more; 4, 6 and 8
+// measured no better).  A group's scales are copied with its operands and
+// counted on the same barrier.  A slot needs no barrier of its own to be reused: the
 // producer writes group i + kSideSlots once the MMA of group i + kSideSlots -
 // kStages is done, which was issued after the epilogue had released group
 // i + kSideSlots - kStages - 2, a group after i.
 constexpr int kOutBlockBytes = 32 * 128;  // 32 rows of 64 two-byte outputs
-template <int NSIDE, bool STAGED>
+//
+// With zero points (ZERO) a stage also holds its group's records as rows of 16
+// bytes, the upper halves zero, 128 of activations and 256 of weights, and a
+// zero block stands for the second 16 bytes of K of both.
+constexpr int kRecRow = 16;
+constexpr int kRecBytes = (BM + BN) * kRecRow;
+template <bool ZERO, bool STAGED>
 struct Smem {
-    static constexpr int kStages = 5;
-    static constexpr int kSideSlots = NSIDE == 1 ? 16 : 8;
+    static constexpr int kStages = ZERO ? 4 : 5;
+    static constexpr int kSideSlots = ZERO ? 8 : 16;
+    static constexpr int kStageBytes = kABytes + kBBytes + (ZERO ? kRecBytes : 0);
+    static constexpr int kRecA = kABytes + kBBytes, kRecW = kRecA + BM * kRecRow;  // in a stage
     static_assert(kSideSlots >= kStages + 3, "a slot is rewritten only after its group's epilogue");
     static constexpr int kOperands = 0;
     static constexpr int kOut = kStages * kStageBytes;
     static constexpr int kSide = kOut + (STAGED ? kEpiWarps * kOutBlockBytes : 0);
-    static constexpr int kSideABytes = NSIDE * BM * 4;
-    static constexpr int kSideSlotBytes = NSIDE * (BM + BN) * 4;
-    static constexpr int kBars = kSide + kSideSlots * kSideSlotBytes;
+    static constexpr int kSideABytes = BM * 4;
+    static constexpr int kSideSlotBytes = (BM + BN) * 4;
+    static constexpr int kZeros = kSide + kSideSlots * kSideSlotBytes;
+    static constexpr int kZeroBytes = ZERO ? BN * kRecRow : 0;
+    static constexpr int kBars = kZeros + kZeroBytes;
     // full, empty, acc_full x2, acc_empty x2, drain
     static constexpr int kNumBars = 2 * kStages + 4 + 1;
     static constexpr int kMisc = kBars + kNumBars * 8;
@@ -616,9 +666,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const GemmArgs args)
 {
     griddep_wait();
-    constexpr int NSIDE = (MODE == QUARTZ_ASYMMETRIC) ? 3 : 1;
-    using L = Smem<NSIDE, OUT != QUARTZ_OUT_F32>;
-    constexpr int kStages = L::kStages;
+    constexpr bool ZERO = MODE == QUARTZ_ASYMMETRIC && !DUMP;  // zero-point terms by the tensor core
+    using L = Smem<ZERO, OUT != QUARTZ_OUT_F32>;
+    constexpr int kStages = L::kStages, kStageBytes = L::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
@@ -636,7 +686,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(full_bar(s), 1);
+            mbar_init(full_bar(s), ZERO ? 2 : 1);  // the copies, and the records
             mbar_init(empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -646,6 +696,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(drain_bar, 1);
         *abort_flag = 0;
         fence_mbar_init();
+    }
+    if constexpr (ZERO) {
+        // the upper halves of the record rows and the zero block stay zero
+        for (int i = threadIdx.x; i < L::kZeroBytes / 16; i += kThreads)
+            *reinterpret_cast<uint4 *>(smem + L::kZeros + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+        for (int st = 0; st < kStages; ++st)
+            for (int i = threadIdx.x; i < kRecBytes / 16; i += kThreads)
+                *reinterpret_cast<uint4 *>(smem + st * kStageBytes + L::kRecA + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async();
     }
     if (warp == kMmaWarp) {
         tmem_alloc(smem_u32(tmem_holder), kTmemCols);
@@ -673,7 +732,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         // from a divergent lane.
         // ------------------------------------------------------------------
         const bool leader = elect_one();
-        const int64_t a_plane = args.m_pad * G, w_plane = args.n_pad * G;
         int it = 0, s = 0;   // groups whose operand copies were issued; the next stage
         uint32_t phase = 1;  // parity of that stage's last release (the first round waits for none)
         bool ok = true;
@@ -691,16 +749,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 if (leader) {
                     const uint32_t sa = smem_base + L::kOperands + s * kStageBytes;
-                    mbar_arrive_expect_tx(full_bar(s), kStageBytes + (PERROW ? 0 : L::kSideSlotBytes));
+                    mbar_arrive_expect_tx(full_bar(s), kABytes + kBBytes + (PERROW ? 0 : L::kSideSlotBytes));
                     tma_load_2d(sa, &tmap_a, g * BK, mt * BM, full_bar(s));
                     tma_load_2d(sa + kABytes, &tmap_w, g * BK, nt * BN, full_bar(s));
                     if (!PERROW) {
                         const uint32_t dst = smem_base + L::kSide + (it % L::kSideSlots) * L::kSideSlotBytes;
-#pragma unroll
-                        for (int sd = 0; sd < NSIDE; ++sd) {
-                            bulk_load(dst + sd * BM * 4, src_a + sd * a_plane, BM * 4, full_bar(s));
-                            bulk_load(dst + L::kSideABytes + sd * BN * 4, src_w + sd * w_plane, BN * 4, full_bar(s));
-                        }
+                        bulk_load(dst, src_a, BM * 4, full_bar(s));
+                        bulk_load(dst + L::kSideABytes, src_w, BN * 4, full_bar(s));
                     }
                 }
                 __syncwarp();
@@ -722,6 +777,60 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         __syncwarp();
+      } else if (ZERO && warp == kRecWarp) {
+        // ------------------------------------------------------------------
+        // Zero-point records: each group's 128 + 256 records go by 8-byte
+        // asynchronous copies into the lower halves of the stage's rows,
+        // kRecDepth groups in flight; a group is handed over once its copies
+        // have landed and are visible to the async proxy.
+        // ------------------------------------------------------------------
+        int it = 0, s = 0, done = 0;  // groups issued, the next stage, the stage to hand over next
+        uint32_t phase = 1;
+        bool ok = true;
+        const int n_items = work_items(args);
+        for (int k = 0; k < n_items && ok; ++k) {
+            const WorkItem wi = work_item(args, k);
+            int mt, nt;
+            tile_coords<RM>(wi.tile, args, mt, nt);
+            const ZeroRec *src_a = zero_recs(args.a_side, G, args.m_pad) + wi.g0 * args.m_pad +
+                                   static_cast<int64_t>(mt) * BM + lane;
+            const ZeroRec *src_w = zero_recs(args.w_side, G, args.n_pad) + wi.g0 * args.n_pad +
+                                   static_cast<int64_t>(nt) * BN + lane;
+            for (int g = wi.g0; g < wi.g1; ++g, ++it) {
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, args.dev_err, kWaitLimitNs)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t dst = smem_base + s * kStageBytes + L::kRecA + lane * kRecRow;
+#pragma unroll
+                for (int i = 0; i < BM / 32; ++i) cp_async8(dst + 32 * i * kRecRow, src_a + 32 * i);
+#pragma unroll
+                for (int i = 0; i < BN / 32; ++i) cp_async8(dst + (BM + 32 * i) * kRecRow, src_w + 32 * i);
+                cp_async_commit();
+                src_a += args.m_pad;
+                src_w += args.n_pad;
+                if (it >= kRecDepth - 1) {
+                    cp_async_wait<kRecDepth - 1>();  // group it - (kRecDepth - 1) has landed
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full_bar(done));
+                    if (++done == kStages) done = 0;
+                }
+                if (++s == kStages) {
+                    s = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+        cp_async_wait<0>();
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0 && ok)
+            for (int i = min(it, kRecDepth - 1); i > 0; --i) {
+                mbar_arrive(full_bar(done));
+                if (++done == kStages) done = 0;
+            }
+        __syncwarp();
       } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------------
         // MMA issuer: 2 x (M=128, N=256, K=32) kind::f8f6f4 MMAs per group into
@@ -732,6 +841,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t idesc = args.wide ? idesc_e5m2_f32(BM, BN) : idesc_e4m3_f32(BM, BN);
             const uint64_t desc_a0 = sdesc_k_major_sw64(smem_base + L::kOperands);
             const uint64_t desc_w0 = sdesc_k_major_sw64(smem_base + L::kOperands + kABytes);
+            // records: 8-row blocks of 16-byte rows 128 bytes apart, the second
+            // 16 bytes of K in the zero block
+            const uint64_t desc_ra0 = sdesc_k_major_none(smem_base + L::kRecA, smem_base + L::kZeros);
+            const uint64_t desc_rw0 = sdesc_k_major_none(smem_base + L::kRecW, smem_base + L::kZeros);
             const bool leader = elect_one();
             int s = 0;
             uint32_t phase = 0;
@@ -758,6 +871,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                         for (int kk = 0; kk < BK / 32; ++kk)
                             mma_f8_ss(tmem_base + static_cast<uint32_t>(b * BN), desc_a0 + st + 2 * kk,
                                       desc_w0 + st + 2 * kk, idesc, (kk > 0 || !first) ? 1u : 0u);
+                        if (ZERO)  // (the distance to the zero block shrinks as the address grows)
+                            mma_f16_ss(tmem_base + static_cast<uint32_t>(b * BN), desc_ra0 + st - (st << 16),
+                                       desc_rw0 + st - (st << 16), idesc_f16_f32(BM, BN), 1u);
                         mma_commit(empty_bar(s));
                         if (last) {
                             mma_commit(acc_full_bar(b));
@@ -794,8 +910,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         // rows) and the stores are 4-wide.  The thread's four row scales are
         // one 16-byte load as well (rows are permuted in the side values).
         // Per group, y += s_a * (s_w * P_g) on (row, row + 8) pairs with
-        // f32x2 arithmetic (asymmetric first adds the exact integer
-        // zero-point terms to P_g).
+        // f32x2 arithmetic (with zero points the tensor core has added their
+        // exact integer terms to P_g).
         // ------------------------------------------------------------------
         const int quarter = warp & 3;
         const int slot = warp >> 2;
@@ -881,8 +997,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 out.end();
             }
-        } else if constexpr (MODE == QUARTZ_SYMMETRIC && !DUMP) {
-            // Symmetric fast path: each half chunk (16 lanes x 16 columns: TMEM
+        } else if constexpr (!DUMP) {
+            // Fast path (with zero points the accumulator holds the corrected
+            // sum): each half chunk (16 lanes x 16 columns: TMEM
             // load, wait and the scale arithmetic) is one PTX block on
             // explicit 64-bit pairs, which keeps the kernel free of spills.
             // The group loop carries only its accumulators, three offsets and
@@ -997,6 +1114,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 out.end();
             }
         } else {
+            // Partials dump: raw P_g, zero-point terms from global memory.
             float2 acc[2][16];
             int it = 0;
             bool ok = true;
@@ -1015,16 +1133,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ok = false;
                         break;
                     }
-                    // cur_a[sd][k]: side value sd of row trow + 8k of the quarter
-                    float cur_a[NSIDE][4];
+                    int mt, nt;
+                    tile_coords<RM>(tile, args, mt, nt);
+                    const int64_t m0 = static_cast<int64_t>(mt) * BM + quarter * 32 + trow;
+                    const int64_t n0 = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + tq;
+                    const float4 sav = lds_f4(side_a);  // scales of rows trow + 8k of the quarter
+                    const float cur_a[4] = {sav.x, sav.y, sav.z, sav.w};
+                    float2 za_u[4];  // (z_a, 64 z_a - A_g) of the same rows
 #pragma unroll
-                    for (int sd = 0; sd < NSIDE; ++sd) {
-                        const float4 v = lds_f4(side_a + sd * BM * 4);
-                        cur_a[sd][0] = v.x;
-                        cur_a[sd][1] = v.y;
-                        cur_a[sd][2] = v.z;
-                        cur_a[sd][3] = v.w;
-                    }
+                    for (int k = 0; k < 4; ++k)
+                        za_u[k] = MODE == QUARTZ_ASYMMETRIC
+                                      ? zero_terms(zero_recs(args.a_side, G, args.m_pad)[g * args.m_pad + m0 + 8 * k], true)
+                                      : make_float2(0.f, 0.f);
                     tc_fence_after();
                     const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
                                            static_cast<uint32_t>(b * BN + slot * kColsPerWarp);
@@ -1035,36 +1155,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tmem_wait_ld(r);
                         const float4 sw = lds_f4(side_w + 16 * chunk * 4);
                         const float swv[4] = {sw.x, sw.y, sw.z, sw.w};
-                        float4 zw4 = make_float4(0.f, 0.f, 0.f, 0.f), gw4 = zw4;
-                        if (MODE == QUARTZ_ASYMMETRIC) {
-                            zw4 = lds_f4(side_w + (BN + 16 * chunk) * 4);
-                            gw4 = lds_f4(side_w + (2 * BN + 16 * chunk) * 4);
-                        }
-                        const float zwv[4] = {zw4.x, zw4.y, zw4.z, zw4.w};
-                        const float gwv[4] = {gw4.x, gw4.y, gw4.z, gw4.w};
+                        float2 zg[4];  // (z_w, W_g) of the four columns
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            zg[i] = MODE == QUARTZ_ASYMMETRIC
+                                        ? zero_terms(zero_recs(args.w_side, G, args.n_pad)[g * args.n_pad + perm16(n0 + 16 * chunk + i)], false)
+                                        : make_float2(0.f, 0.f);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 float2 p = make_float2(__uint_as_float(r[8 * h + 2 * i]), __uint_as_float(r[8 * h + 2 * i + 1]));
                                 if (DUMP && g == args.partials_group) {
-                                    int mt, nt;
-                                    tile_coords<RM>(tile, args, mt, nt);
-                                    const int64_t m = static_cast<int64_t>(mt) * BM + quarter * 32 + 16 * h + trow;
-                                    const int64_t n = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + 16 * chunk + tq + i;
+                                    const int64_t m = m0 + 16 * h, n = n0 + 16 * chunk + i;
                                     if (n < args.N) {
                                         if (m < args.M) args.partials[m * args.N + n] = __float2int_rn(p.x);
                                         if (m + 8 < args.M) args.partials[(m + 8) * args.N + n] = __float2int_rn(p.y);
                                     }
                                 }
                                 if (MODE == QUARTZ_ASYMMETRIC) {
-                                    const float2 ua = make_float2(cur_a[2][2 * h], cur_a[2][2 * h + 1]);
-                                    const float2 nza = make_float2(-cur_a[1][2 * h], -cur_a[1][2 * h + 1]);
-                                    p = __ffma2_rn(make_float2(zwv[i], zwv[i]), ua, p);
-                                    p = __ffma2_rn(nza, make_float2(gwv[i], gwv[i]), p);
+                                    const float2 ua = make_float2(za_u[2 * h].y, za_u[2 * h + 1].y);
+                                    const float2 nza = make_float2(-za_u[2 * h].x, -za_u[2 * h + 1].x);
+                                    p = __ffma2_rn(make_float2(zg[i].x, zg[i].x), ua, p);
+                                    p = __ffma2_rn(nza, make_float2(zg[i].y, zg[i].y), p);
                                 }
                                 const float2 t = __fmul2_rn(p, make_float2(swv[i], swv[i]));
-                                acc[h][4 * chunk + i] = __ffma2_rn(t, make_float2(cur_a[0][2 * h], cur_a[0][2 * h + 1]),
+                                acc[h][4 * chunk + i] = __ffma2_rn(t, make_float2(cur_a[2 * h], cur_a[2 * h + 1]),
                                                                    acc[h][4 * chunk + i]);
                             }
                         }
@@ -1181,8 +1297,6 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const __nv_fp8_e4m3 *__r
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
     float y[4][4] = {};
-    const int64_t a_plane = args.m_pad * args.G;
-    const int64_t w_plane = args.n_pad * args.G;
     for (int g = 0; g < args.G; ++g) {
         for (int i = threadIdx.x; i < 64 * kGroupQ; i += 256) {
             const int r = i / kGroupQ, k = i % kGroupQ;
@@ -1208,12 +1322,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const __nv_fp8_e4m3 *__r
                 float P = static_cast<float>(p[i][j]);
                 if (args.partials && g == args.partials_group) args.partials[(int64_t)m * args.N + n] = p[i][j];
                 if (MODE == QUARTZ_ASYMMETRIC) {
-                    const float za = args.a_side[a_plane + (int64_t)g * args.m_pad + perm32(m)];
-                    const float ua = args.a_side[2 * a_plane + (int64_t)g * args.m_pad + perm32(m)];
-                    const float zw = args.w_side[w_plane + (int64_t)g * args.n_pad + n];
-                    const float gw = args.w_side[2 * w_plane + (int64_t)g * args.n_pad + n];
-                    P = __fmaf_rn(zw, ua, P);
-                    P = __fmaf_rn(-za, gw, P);
+                    const float2 ta = zero_terms(zero_recs(args.a_side, args.G, args.m_pad)[(int64_t)g * args.m_pad + m], true);
+                    const float2 tw =
+                        zero_terms(zero_recs(args.w_side, args.G, args.n_pad)[(int64_t)g * args.n_pad + perm16(n)], false);
+                    P = __fmaf_rn(tw.x, ta.y, P);
+                    P = __fmaf_rn(-ta.x, tw.y, P);
                 }
                 const float t = __fmul_rn(P, args.w_side[static_cast<int64_t>(g) * args.n_pad + n]);
                 y[i][j] = __fmaf_rn(t, s_a, y[i][j]);
@@ -1269,8 +1382,6 @@ __global__ void __launch_bounds__(256) gemm_shift_kernel(const uint32_t *__restr
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
     const int64_t words_per_row = K / 8, flags_per_row = K / GS;
     float y[4][4] = {};
-    const int64_t a_plane = args.m_pad * args.G;
-    const int64_t w_plane = args.n_pad * args.G;
     for (int g = 0; g < args.G; ++g) {
         for (int i = threadIdx.x; i < 64 * (kGroupQ / 8); i += 256) {
             const int r = i / (kGroupQ / 8), wi = i % (kGroupQ / 8);
@@ -1318,12 +1429,11 @@ __global__ void __launch_bounds__(256) gemm_shift_kernel(const uint32_t *__restr
                 if (!WIDE && args.partials && g == args.partials_group)
                     args.partials[(int64_t)m * args.N + n] = static_cast<int32_t>(p[i][jj]);
                 if (MODE == QUARTZ_ASYMMETRIC) {
-                    const float za = args.a_side[a_plane + (int64_t)g * args.m_pad + perm32(m)];
-                    const float ua = args.a_side[2 * a_plane + (int64_t)g * args.m_pad + perm32(m)];
-                    const float zw = args.w_side[w_plane + (int64_t)g * args.n_pad + n];
-                    const float gw = args.w_side[2 * w_plane + (int64_t)g * args.n_pad + n];
-                    P = __fmaf_rn(zw, ua, P);
-                    P = __fmaf_rn(-za, gw, P);
+                    const float2 ta = zero_terms(zero_recs(args.a_side, args.G, args.m_pad)[(int64_t)g * args.m_pad + m], true);
+                    const float2 tw =
+                        zero_terms(zero_recs(args.w_side, args.G, args.n_pad)[(int64_t)g * args.n_pad + perm16(n)], false);
+                    P = __fmaf_rn(tw.x, ta.y, P);
+                    P = __fmaf_rn(-ta.x, tw.y, P);
                 }
                 const float t = __fmul_rn(P, args.w_side[static_cast<int64_t>(g) * args.n_pad + n]);
                 y[i][jj] = __fmaf_rn(t, s_a, y[i][jj]);
@@ -1431,9 +1541,10 @@ template <int MODE, int OUT>
 cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &ty, const GemmArgs &args,
                       cudaStream_t s)
 {
-    constexpr int NSIDE = (MODE == QUARTZ_ASYMMETRIC) ? 3 : 1;
-    constexpr int smem = Smem<NSIDE, OUT != QUARTZ_OUT_F32>::kAlloc;
-    static_assert(smem <= 227 * 1024, "shared memory budget");
+    constexpr bool staged = OUT != QUARTZ_OUT_F32;
+    static_assert(Smem<true, staged>::kAlloc <= 227 * 1024 && Smem<false, staged>::kAlloc <= 227 * 1024,
+                  "shared memory budget");
+    const int smem = MODE == QUARTZ_ASYMMETRIC && !args.partials ? Smem<true, staged>::kAlloc : Smem<false, staged>::kAlloc;
     auto kern = args.partials ? gemm_tcgen05_kernel<MODE, OUT, true, false>
                               : gemm_tcgen05_kernel<MODE, OUT, false, false>;
     if constexpr (MODE == QUARTZ_SYMMETRIC) {

@@ -179,6 +179,15 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 // async proxy (TMA, tcgen05).
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// 8-byte asynchronous copy global -> shared by this thread, in commit groups.
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // 2-D tiled tensor store shared -> global, tracked by this thread's bulk
 // groups; parts of the box outside the tensor are not written.
 __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t src, int32_t x, int32_t y)
@@ -247,6 +256,37 @@ __device__ __forceinline__ uint64_t sdesc_k_major_sw64(uint32_t addr)
     d |= (uint64_t)1u << 46;
     d |= (uint64_t)4u << 61;                          // swizzle: 64B
     return d;
+}
+
+// Shared-memory matrix descriptor of K-major rows of 16 bytes without swizzle:
+// 8-row blocks 128 bytes apart (stride byte offset); the second 16 bytes of K
+// lie at `next` (leading byte offset, above `addr`).
+__device__ __forceinline__ uint64_t sdesc_k_major_none(uint32_t addr, uint32_t next)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)((next - addr) >> 4) << 16;
+    d |= (uint64_t)(128u >> 4) << 32;
+    d |= (uint64_t)1u << 46;
+    return d;
+}
+
+// The MMA below with fp16 A and B (K = 16).
+__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                           uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Instruction descriptor of kind::f16: fp16 A and B (format 0, K-major), fp32 D.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(uint32_t M, uint32_t N)
+{
+    return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
 // D (TMEM, fp32) = A * B (+ D if `accumulate`), A and B FP8 from shared memory.

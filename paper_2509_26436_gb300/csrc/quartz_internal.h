@@ -80,8 +80,8 @@ __host__ __device__ __forceinline__ int64_t perm32(int64_t r)
 struct LinearWorkspace {
     void *a_op;      // E4M3 [M, K]  decoded activations
     void *w_op;      // E4M3 [round_up(N, 16), K]  decoded weights, rows transposed 4x4 inside 16-row blocks
-    float *a_side;   // fp32 [nside][G][Mpad]  scale (and z, gsum when asymmetric)
-    float *w_side;   // fp32 [nside][G][Npad]
+    float *a_side;   // fp32 [G][Mpad] scales; asymmetric: then 8-byte zero-point records [G][Mpad] (linear.cu: ZeroRec)
+    float *w_side;   // the same [G][Npad]
     float *tail_part;  // fp32 partial tiles of the split last wave (may be NULL)
     int64_t m_pad, n_pad;
     int nside;
