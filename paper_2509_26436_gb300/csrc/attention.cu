@@ -32,6 +32,18 @@
 //     CTAs fit an SM); FLAGs and scales of the next tile are prefetched
 //     into registers.  Output per CTA: unnormalised o, running
 //     max, running sum.
+//     What bounds it: instruction issue as much as memory.  A 128-token tile
+//     took 842 instructions a warp (32 x 16 heads, 4096 tokens, G_s = 16:
+//     issue slots 67% busy, the half-rate ALU 63%, DRAM 56%), of which the
+//     unpack and the multiply-adds of the values need some 300.  So the rest
+//     is kept small: addresses are a base per CTA plus 32-bit offsets, a full
+//     tile is copied without row checks, the FLAG form (bytes or nibbles) is a
+//     template argument, and a key's FLAG shifts the 16-fold dot product,
+//     which is divided by 16 once per 64-wide group.  72.7 -> 64.7 us there,
+//     80.7 -> 71.4 at G_s = 8, 68.4 -> 65.8 at G_s = 32, 131 -> 116 with 64 x
+//     16 heads.  Measured and not used: independent warps without CTA barriers
+//     (+-3%); the tiles of all heads cut into equal runs, one wave of CTAs
+//     (0-8% slower).
 //   attn_combine_kernel: one CTA per bh merges the splits.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -72,8 +84,8 @@ struct AttnArgs {
 
 // The FLAG bytes (or nibbles) of one token row: S = 128 / G_s subgroups,
 // stored at subgroup index row * S + j (one byte each, or two per byte).
-template <int GS>
-__device__ __forceinline__ void load_row_flags(const uint8_t *flags, int64_t row, bool packed, uint32_t (&f)[4])
+template <int GS, typename Row>
+__device__ __forceinline__ void load_row_flags(const uint8_t *flags, Row row, bool packed, uint32_t (&f)[4])
 {
     constexpr int S = kD / GS;
     f[0] = f[1] = f[2] = f[3] = 0u;
@@ -100,7 +112,8 @@ __device__ __forceinline__ int row_flag(const uint32_t (&f)[4], int j, bool pack
                   : static_cast<int>((f[j >> 2] >> (8 * (j & 3))) & 0xFFu);
 }
 
-__device__ __forceinline__ float2 load_scales2(const __half *scales, int64_t row)
+template <typename Row>
+__device__ __forceinline__ float2 load_scales2(const __half *scales, Row row)
 {
     const uint32_t w = *reinterpret_cast<const uint32_t *>(scales + 2 * row);
     return __half22float2(*reinterpret_cast<const __half2 *>(&w));
@@ -164,14 +177,23 @@ struct RowSide {
     float2 sk, sv;
 };
 
-template <int GS>
-__device__ __forceinline__ void load_side(const AttnArgs &a, int64_t row, bool valid, RowSide &r)
+// The four arrays at a CTA's first token (uniform addresses), so that a
+// thread's loads need a 32-bit token offset only.
+struct SideBase {
+    const uint8_t *kf, *vf;
+    const __half *ks, *vs;
+};
+
+// PACK: 0 = one FLAG byte per subgroup in both caches, 1 = 4-bit FLAGs in
+// both, -1 = as the arguments say (the caches differ).
+template <int GS, int PACK>
+__device__ __forceinline__ void load_side(const AttnArgs &a, const SideBase &b, uint32_t t, bool valid, RowSide &r)
 {
     if (valid) {
-        load_row_flags<GS>(a.k_flags, row, a.k_packed != 0, r.kf);
-        load_row_flags<GS>(a.v_flags, row, a.v_packed != 0, r.vf);
-        r.sk = load_scales2(a.k_scales, row);
-        r.sv = load_scales2(a.v_scales, row);
+        load_row_flags<GS>(b.kf, t, PACK < 0 ? a.k_packed != 0 : PACK, r.kf);
+        load_row_flags<GS>(b.vf, t, PACK < 0 ? a.v_packed != 0 : PACK, r.vf);
+        r.sk = load_scales2(b.ks, t);
+        r.sv = load_scales2(b.vs, t);
     } else {
         r.kf[0] = r.kf[1] = r.kf[2] = r.kf[3] = 0u;
         r.vf[0] = r.vf[1] = r.vf[2] = r.vf[3] = 0u;
@@ -201,7 +223,7 @@ static_assert(kAttnThreads * (16 + 1) * 4 <= kAttnDynSmem && kAttnThreads * (32 
 template <int GS>
 constexpr int attn_min_ctas() { return GS == 16 || GS == 32 ? 6 : 5; }
 
-template <int GS>
+template <int GS, int PACK>
 __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode_kernel(const __grid_constant__ AttnArgs a)
 {
     griddep_wait();
@@ -220,24 +242,34 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     const int t_end = min(t_begin + a.chunk, a.L);
     const int n_tiles = (t_end - t_begin + kTile - 1) / kTile;
     const uint32_t ring = static_cast<uint32_t>(__cvta_generic_to_shared(s_ring));
-    const uint8_t *kbytes = reinterpret_cast<const uint8_t *>(a.k_codes);
-    const uint8_t *vbytes = reinterpret_cast<const uint8_t *>(a.v_codes);
+    const bool k_packed = PACK < 0 ? a.k_packed != 0 : PACK, v_packed = PACK < 0 ? a.v_packed != 0 : PACK;
+    const int n_tok = t_end - t_begin;
+    const int64_t row0 = bh * a.L_max + t_begin;  // the CTA's first token in the caches
+    const SideBase side = {a.k_flags + row0 * (k_packed ? S / 2 : S), a.v_flags + row0 * (v_packed ? S / 2 : S),
+                           a.k_scales + 2 * row0, a.v_scales + 2 * row0};
+    // this thread's chunks of a code tile: rows tid / 4 + 32 k, whose swizzle is the same for every k
+    const uint8_t *kbytes = reinterpret_cast<const uint8_t *>(a.k_codes) + row0 * (kD / 2);
+    const uint8_t *vbytes = reinterpret_cast<const uint8_t *>(a.v_codes) + row0 * (kD / 2);
+    const uint32_t ring_dst = ring + tile_off(tid >> 2, tid & 3);
 
     // Copies of tile `it` (both caches) into stage it % kStages; every thread
     // commits one group per call, empty past the last tile.
     auto issue = [&](int it) {
-        if (it < n_tiles) {
-            const int tile = t_begin + it * kTile;
-            const uint32_t kdst = ring + (it % kStages) * 2 * kTileBytes;
-            const uint32_t vdst = kdst + kTileBytes;
+        const int left = n_tok - it * kTile;  // tokens from this tile on
+        const uint32_t kdst = ring_dst + (it % kStages) * 2 * kTileBytes;
+        const uint32_t src = static_cast<uint32_t>(it) * kTileBytes + tid * 16;
+        if (left >= kTile) {
 #pragma unroll
             for (int k = 0; k < kTileBytes / 16 / kAttnThreads; ++k) {
-                const int ci = tid + k * kAttnThreads;
-                const int r = ci >> 2, c = ci & 3;
-                if (tile + r < t_end) {
-                    const int64_t src = (bh * a.L_max + tile + r) * (kD / 2) + c * 16;
-                    cp_async16(kdst + tile_off(r, c), kbytes + src);
-                    cp_async16(vdst + tile_off(r, c), vbytes + src);
+                cp_async16(kdst + k * kAttnThreads * 16, kbytes + src + k * kAttnThreads * 16);
+                cp_async16(kdst + kTileBytes + k * kAttnThreads * 16, vbytes + src + k * kAttnThreads * 16);
+            }
+        } else if (left > 0) {
+#pragma unroll
+            for (int k = 0; k < kTileBytes / 16 / kAttnThreads; ++k) {
+                if ((tid >> 2) + k * (kAttnThreads / 4) < left) {
+                    cp_async16(kdst + k * kAttnThreads * 16, kbytes + src + k * kAttnThreads * 16);
+                    cp_async16(kdst + kTileBytes + k * kAttnThreads * 16, vbytes + src + k * kAttnThreads * 16);
                 }
             }
         }
@@ -266,7 +298,7 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     }
     const float2 sq = load_scales2(a.q_scales, bh);
     RowSide cur;
-    load_side<GS>(a, bh * a.L_max + t_begin + tid, t_begin + tid < t_end, cur);
+    load_side<GS, PACK>(a, side, tid, tid < n_tok, cur);
     __syncthreads();
     const uint32_t sq_addr = static_cast<uint32_t>(__cvta_generic_to_shared(s_q));
 
@@ -276,6 +308,13 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     constexpr int kWordsPerPiece = kValDims / 8;       // 32-bit code words per piece
     const int vc = tid % kPieces;   // value phase: code piece (dims kValDims vc ..)
     const int slot = tid / kPieces; // value phase: token slot
+    // offsets in a code tile: the thread's key row, and its value piece of token `slot`
+    // (the swizzle is the same for tokens slot + i kSlots)
+    static_assert(kSlots % 8 == 0, "the swizzle repeats every 8 rows");
+    uint32_t key_off[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) key_off[c] = tile_off(tid, c);
+    const uint32_t val_off = kWordsPerPiece == 4 ? tile_off(slot, vc) : tile_off(slot, vc >> 1) + 8 * (vc & 1);
     float acc[kValDims];
 #pragma unroll
     for (int k = 0; k < kValDims; ++k) acc[k] = 0.f;
@@ -283,7 +322,6 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     float l_thr = 0.f;        // this thread's share of the running sum
 
     for (int it = 0; it < n_tiles; ++it) {
-        const int tile = t_begin + it * kTile;
         issue(it + kStages - 1);     // into the stage tile it - 1 used
         cp_async_wait<kStages - 1>();  // this thread's copies of tile `it` have landed
         __syncthreads();     // ... and everyone else's
@@ -291,16 +329,17 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
         const uint32_t vst = kst + kTileBytes;
         // FLAGs and scales of the next tile, while this one is processed
         RowSide nxt;
-        load_side<GS>(a, bh * a.L_max + tile + kTile + tid, tile + kTile + tid < t_end, nxt);
+        const int t_next = (it + 1) * kTile + tid;
+        load_side<GS, PACK>(a, side, static_cast<uint32_t>(t_next), t_next < n_tok, nxt);
 
         // ---- keys: one token per thread -----------------------------------
-        const bool valid = tile + tid < t_end;
+        const bool valid = it * kTile + tid < n_tok;
         float s2 = -INFINITY;
         if (valid) {
             uint32_t kw[kWords], qe[kWords], qo[kWords];  // the query words: broadcast shared loads
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const uint4 v = lds_u4(kst + tile_off(tid, c));
+                const uint4 v = lds_u4(kst + key_off[c]);
                 kw[4 * c] = v.x, kw[4 * c + 1] = v.y, kw[4 * c + 2] = v.z, kw[4 * c + 3] = v.w;
                 const uint4 e = lds_u4(sq_addr + 16 * c);
                 qe[4 * c] = e.x, qe[4 * c + 1] = e.y, qe[4 * c + 2] = e.z, qe[4 * c + 3] = e.w;
@@ -316,10 +355,10 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
                     dot = __dp4a(static_cast<int>(qe[w]), static_cast<int>((kw[w] << 4) & 0xF0F0F0F0u), dot);
                     dot = __dp4a(static_cast<int>(qo[w]), static_cast<int>(kw[w] & 0xF0F0F0F0u), dot);
                 }
-                P[(j * GS) / 64] += (dot >> 4) * (1 << row_flag(cur.kf, j, a.k_packed != 0));
+                P[(j * GS) / 64] += dot << row_flag(cur.kf, j, k_packed);  // 16 x the group sum, in 27 bits
             }
-            const float sc = __fmul_rn(__fmul_rn(sq.x, cur.sk.x), static_cast<float>(P[0])) +
-                             __fmul_rn(__fmul_rn(sq.y, cur.sk.y), static_cast<float>(P[1]));
+            const float sc = __fmul_rn(__fmul_rn(sq.x, cur.sk.x), static_cast<float>(P[0] >> 4)) +
+                             __fmul_rn(__fmul_rn(sq.y, cur.sk.y), static_cast<float>(P[1] >> 4));
             s2 = sc * a.scale_log2;
         }
 
@@ -338,7 +377,7 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
         l_thr = l_thr * alpha + p;
 #pragma unroll
         for (int j = 0; j < S; ++j)  // p_t s_v 2^FLAG of every value subgroup (0 past the end)
-            s_pf[j][tid] = p * scale_pow2((j * GS) / 64 ? cur.sv.y : cur.sv.x, row_flag(cur.vf, j, a.v_packed != 0));
+            s_pf[j][tid] = p * scale_pow2((j * GS) / 64 ? cur.sv.y : cur.sv.x, row_flag(cur.vf, j, v_packed));
         if (m_new != m_run) {  // CTA-uniform: rescale only when the maximum grew
 #pragma unroll
             for (int k = 0; k < kValDims; ++k) acc[k] *= alpha;
@@ -352,11 +391,11 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
             const int ti = slot + i * kSlots;
             uint32_t words[kWordsPerPiece];
             if constexpr (kWordsPerPiece == 4) {
-                const uint4 ch = lds_u4(vst + tile_off(ti, vc));
+                const uint4 ch = lds_u4(vst + val_off + i * kSlots * 64);
                 words[0] = ch.x, words[1] = ch.y, words[2] = ch.z, words[3] = ch.w;
             } else {
                 asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(words[0]), "=r"(words[1])
-                             : "r"(vst + tile_off(ti, vc >> 1) + 8 * (vc & 1)));
+                             : "r"(vst + val_off + i * kSlots * 64));
             }
 #pragma unroll
             for (int w = 0; w < kWordsPerPiece; ++w) {
@@ -444,19 +483,19 @@ int attn_splits(int64_t BH, int64_t L, int64_t slots, int *chunk)
     return static_cast<int>((tiles + per - 1) / per);
 }
 
-template <int GS>
+template <int GS, int PACK>
 cudaError_t launch_decode(int64_t BH, AttnArgs &a, cudaStream_t s)
 {
     // resident CTAs per SM of this instance, looked up on first use (any
     // host thread; they all store the same value)
     static std::atomic<int> occ_cache{0};
-    cudaError_t e = cudaFuncSetAttribute(attn_decode_kernel<GS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(attn_decode_kernel<GS, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kAttnDynSmem);
     if (e != cudaSuccess) return e;
     int occ = occ_cache.load(std::memory_order_relaxed);
     if (occ == 0) {
         int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attn_decode_kernel<GS>, kAttnThreads, kAttnDynSmem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attn_decode_kernel<GS, PACK>, kAttnThreads, kAttnDynSmem);
         if (e != cudaSuccess) return e;
         occ = n > 0 ? n : 1;
         occ_cache.store(occ, std::memory_order_relaxed);
@@ -467,8 +506,18 @@ cudaError_t launch_decode(int64_t BH, AttnArgs &a, cudaStream_t s)
     if (sms <= 0) sms = 1;
     a.n_split = attn_splits(BH, a.L, static_cast<int64_t>(sms) * occ, &a.chunk);
     const dim3 grid(static_cast<unsigned>(a.n_split), static_cast<unsigned>(BH));
-    launch_pdl(attn_decode_kernel<GS>, dim3(grid), dim3(kAttnThreads), kAttnDynSmem, s, a);
+    launch_pdl(attn_decode_kernel<GS, PACK>, dim3(grid), dim3(kAttnThreads), kAttnDynSmem, s, a);
     return cudaGetLastError();
+}
+
+// The FLAG form as a template argument: read at run time it cost about five
+// instructions per FLAG and token (both forms extracted, one selected).
+// Caches that differ in it take the instance that reads it from the arguments.
+template <int GS>
+cudaError_t launch_decode(int64_t BH, AttnArgs &a, cudaStream_t s)
+{
+    if (a.k_packed != a.v_packed) return launch_decode<GS, -1>(BH, a, s);
+    return a.k_packed ? launch_decode<GS, 1>(BH, a, s) : launch_decode<GS, 0>(BH, a, s);
 }
 
 }  // namespace
