@@ -21,8 +21,8 @@
 //     accumulator-shift schedule (Section 4.4) on the key side, exact.
 //     Softmax: running maximum and sum per CTA in the log2 domain; each key
 //     thread then writes p_t s_v 2^FLAG for its token's value subgroups
-//     (the FLAG added to the scale's exponent field).  Values: 4 threads per
-//     token row (one 16-byte chunk of 32 codes each) x 32 token slots; each
+//     (the FLAG added to the scale's exponent field).  Values: 8 threads per
+//     token row (one 8-byte piece of 16 codes each) x 16 token slots; each
 //     code becomes a float exactly through the 2^23 magic number, and
 //     o += p_t s_v 2^FLAG c with paired f32x2 subtract and fused
 //     multiply-add (two instructions per two codes).  The code tiles of
@@ -40,7 +40,7 @@
 //     tile is copied without row checks, the FLAG form (bytes or nibbles) is a
 //     template argument, and a key's FLAG shifts the 16-fold dot product,
 //     which is divided by 16 once per 64-wide group.  72.7 -> 64.7 us there,
-//     80.7 -> 71.4 at G_s = 8, 68.4 -> 65.8 at G_s = 32, 131 -> 116 with 64 x
+//     80.7 -> 71.4 at G_s = 8, 68.4 -> 62.4 at G_s = 32 (with the value layout below), 131 -> 116 with 64 x
 //     16 heads.  Measured and not used: independent warps without CTA barriers
 //     (+-3%); the tiles of all heads cut into equal runs, one wave of CTAs
 //     (0-8% slower).
@@ -233,24 +233,20 @@ __device__ __forceinline__ void load_side(const AttnArgs &a, const SideBase &b, 
 constexpr int kStages = 2;                     // code tiles in flight per CTA
 constexpr int kTileBytes = kTile * kD / 2;     // 8 KB of codes per tile and cache
 constexpr int kAttnDynSmem = kStages * 2 * kTileBytes;
-// Value phase layout: each thread takes kValDims dimensions (one piece of
-// a token row's codes) of tile_tokens / slots tokens.  16 dimensions (an
-// 8-byte piece, 16 accumulators) at G_s = 8 and 16: fewer registers, which
-// lets G_s = 16 run 6 CTAs per SM (2-3% faster at G_s = 8 and 16); 32 (a
-// 16-byte chunk) at G_s = 32 and 64, 1% faster there.
-template <int GS>
-constexpr int val_dims() { return GS <= 16 ? 16 : 32; }
-static_assert(kAttnThreads * (16 + 1) * 4 <= kAttnDynSmem && kAttnThreads * (32 + 1) * 4 <= kAttnDynSmem,
-              "slot reduction fits the code ring");
+// Value phase layout: each thread takes kValDims = 16 dimensions (one 8-byte
+// piece of a token row's codes, 16 accumulators) of kTile / kSlots tokens.
+// With 32 dimensions (a 16-byte chunk) the registers of G_s = 32 spilled at
+// 6 CTAs per SM: 65.0 us against 62.4 (32 x 16 heads, 4096 tokens).
+constexpr int kValDims = 16;
+static_assert(kAttnThreads * (kValDims + 1) * 4 <= kAttnDynSmem, "slot reduction fits the code ring");
 
 // Resident CTAs per SM the register allocation is bounded for: more warps
-// cover the memory latency.  5 (at most 102 registers, no spills) measured
-// 8-10% faster than the unbounded 120-register build.  At G_s = 16 and 32
-// the shared memory of 6 CTAs fits and the kernel compiles to at most 80
-// registers without spills (G_s = 16 with the 16-dimension value layout):
-// 3-4% faster; at G_s = 8 shared memory allows only 5.
+// cover the memory latency.  The shared memory of 6 CTAs fits and the kernel
+// compiles to at most 80 registers from G_s = 16 on (3-4% faster than 5, and
+// 5 8-10% faster than an unbounded build; G_s = 64 64.8 -> 63.5 us with 6);
+// at G_s = 8 shared memory allows only 5.
 template <int GS>
-constexpr int attn_min_ctas() { return GS == 16 || GS == 32 ? 6 : 5; }
+constexpr int attn_min_ctas() { return GS >= 16 ? 6 : 5; }
 
 template <int GS, int PACK>
 __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode_kernel(const __grid_constant__ AttnArgs a)
@@ -331,7 +327,6 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     __syncthreads();
     const uint32_t sq_addr = static_cast<uint32_t>(__cvta_generic_to_shared(s_q));
 
-    constexpr int kValDims = val_dims<GS>();          // value phase: dimensions per thread
     constexpr int kPieces = kD / kValDims;             // code pieces per token row
     constexpr int kSlots = kAttnThreads / kPieces;     // token slots
     constexpr int kWordsPerPiece = kValDims / 8;       // 32-bit code words per piece
@@ -343,7 +338,7 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     uint32_t key_off[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) key_off[c] = tile_off(tid, c);
-    const uint32_t val_off = kWordsPerPiece == 4 ? tile_off(slot, vc) : tile_off(slot, vc >> 1) + 8 * (vc & 1);
+    const uint32_t val_off = tile_off(slot, vc >> 1) + 8 * (vc & 1);
     float acc[kValDims];
 #pragma unroll
     for (int k = 0; k < kValDims; ++k) acc[k] = 0.f;
@@ -419,13 +414,8 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
         for (int i = 0; i < kTile / kSlots; ++i) {
             const int ti = slot + i * kSlots;
             uint32_t words[kWordsPerPiece];
-            if constexpr (kWordsPerPiece == 4) {
-                const uint4 ch = lds_u4(vst + val_off + i * kSlots * 64);
-                words[0] = ch.x, words[1] = ch.y, words[2] = ch.z, words[3] = ch.w;
-            } else {
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(words[0]), "=r"(words[1])
-                             : "r"(vst + val_off + i * kSlots * 64));
-            }
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(words[0]), "=r"(words[1])
+                         : "r"(vst + val_off + i * kSlots * 64));
 #pragma unroll
             for (int w = 0; w < kWordsPerPiece; ++w) {
                 // word kWordsPerPiece vc + w of the row; its subgroup's factor (0 past the end)
