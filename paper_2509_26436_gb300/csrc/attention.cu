@@ -518,11 +518,33 @@ __global__ void __launch_bounds__(kD) attn_combine_kernel(const float *__restric
     const int64_t bh = blockIdx.x;
     const int d = threadIdx.x;
     const float *p = part + bh * n_split * kPartStride;
+    // The kernel is all latency.  The first 8 splits' values are loaded
+    // together, not maxima first: 32 x 4 heads with 8 splits 19.6 -> 18.6 us
+    // for the whole step, 32 x 16 heads with 4 splits 64.6 -> 64.1; 4 or 16
+    // instead of 8 measured within 0.3 us at 4 splits, and 4 costs 0.7 at 8.
+    constexpr int kCombine = 8;
+    float m[kCombine], l[kCombine], o[kCombine];
+#pragma unroll
+    for (int s = 0; s < kCombine; ++s) {
+        const bool in = s < n_split;
+        m[s] = in ? p[s * kPartStride + kD] : -INFINITY;
+        l[s] = in ? p[s * kPartStride + kD + 1] : 0.f;
+        o[s] = in ? p[s * kPartStride + d] : 0.f;
+    }
     float M = -INFINITY;
-    for (int s = 0; s < n_split; ++s) M = fmaxf(M, p[s * kPartStride + kD]);
+#pragma unroll
+    for (int s = 0; s < kCombine; ++s) M = fmaxf(M, m[s]);
+    for (int s = kCombine; s < n_split; ++s) M = fmaxf(M, p[s * kPartStride + kD]);
     float num = 0.f, den = 0.f;
-    for (int s = 0; s < n_split; ++s) {
-        const float w = exp2f(p[s * kPartStride + kD] - M);  // 0 for an empty split
+#pragma unroll
+    for (int s = 0; s < kCombine; ++s)
+        if (s < n_split) {
+            const float w = exp2f(m[s] - M);  // 0 for an empty split
+            num = fmaf(w, o[s], num);
+            den = fmaf(w, l[s], den);
+        }
+    for (int s = kCombine; s < n_split; ++s) {
+        const float w = exp2f(p[s * kPartStride + kD] - M);
         num = fmaf(w, p[s * kPartStride + d], num);
         den = fmaf(w, p[s * kPartStride + kD + 1], den);
     }
