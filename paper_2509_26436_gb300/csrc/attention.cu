@@ -40,8 +40,8 @@
 //     tile is copied without row checks, the FLAG form (bytes or nibbles) is a
 //     template argument, and a key's FLAG shifts the 16-fold dot product,
 //     which is divided by 16 once per 64-wide group.  72.7 -> 64.7 us there,
-//     80.7 -> 71.4 at G_s = 8, 68.4 -> 62.4 at G_s = 32 (with the value layout below), 131 -> 116 with 64 x
-//     16 heads.  Measured and not used: independent warps without CTA barriers
+//     80.7 -> 71.4 at G_s = 8, 68.4 -> 62.4 at G_s = 32 (with the value layout
+//     below), 131 -> 116 with 64 x 16 heads.  Measured and not used: independent warps without CTA barriers
 //     (+-3%); the tiles of all heads cut into equal runs, one wave of CTAs
 //     (0-8% slower).
 //   attn_combine_kernel: one CTA per bh merges the splits, where

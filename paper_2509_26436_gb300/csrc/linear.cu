@@ -5,14 +5,14 @@
 //      are decoded to v = sgn(c)(|c| << FLAG) and written as FP8 E4M3 (exact:
 //      every decoded value is |c| <= 7 times a power of two up to 2^4, i.e.
 //      at most 3 significant bits and |v| <= 112, inside E4M3's 4-bit
-//      significand and 448 range), together with the group scales (and
-//      zero-point side values) transposed to [G][rows] fp32 for contiguous
-//      per-group access.  This pass is HBM-bound and touches each operand
+//      significand and 448 range), together with the group scales
+//      transposed to [G][rows] fp32 (and the zero-point terms to records in
+//      the same order, see ZeroRec) for contiguous per-group access.  This pass is HBM-bound and touches each operand
 //      element once, instead of once per output tile that reads it.
 //   2. GEMM: a persistent warp-specialised tcgen05 kernel.  One TMA warp
 //      streams 128x64 A and 256x64 W tiles (one 64-wide quantization group
 //      per stage, 64-byte swizzle) into a 5-stage shared-memory ring, with
-//      each group's scales on the same barrier; one thread issues
+//      each group's scales on the same barrier; one lane issues
 //      kind::f8f6f4 MMAs into a fresh fp32 TMEM accumulator for every group
 //      (double-buffered, 2 x 256 columns), so each accumulator holds exactly
 //      P_g = sum_{k in g} v_a v_w; sixteen epilogue warps read P_g with
@@ -79,8 +79,9 @@ __host__ __device__ __forceinline__ int64_t perm16(int64_t r)
 // its fp32 accumulator, all integers below 2^23, as a K = 16 step of which 4
 // are used.  Against two more fused multiply-adds per output and group in the
 // epilogue (GEMM, CUDA events): 18432 x 3072 x 3072 461 -> 277 us, 4001 x 3456
-// x 1152 53.9 -> 37.5; results are the same bits.  Activation records are stored in row order, weight records in
-// operand order (perm16), the order of the GEMM's accumulator.
+// x 1152 53.9 -> 37.5; results are the same bits.  Activation records are
+// stored in row order, weight records in operand order (perm16), the order of
+// the GEMM's accumulator.
 struct ZeroRec {
     __half v[4];
 };
@@ -261,8 +262,8 @@ constexpr int BK = kGroupQ;
 constexpr int kABytes = BM * BK;      // E4M3 operands: one byte per element
 constexpr int kBBytes = BN * BK;
 // Warpgroups 0-3 dequantise (16 warps: four per 32-lane TMEM quarter, 64
-// columns each); warpgroup 4 holds the TMA producer, the MMA issuer and two
-// idle warps.  The dequant epilogue is the throughput-critical part (two fp32
+// columns each); warpgroup 4 holds the TMA producer, the MMA issuer, the
+// zero-point record warp and an idle one.  The dequant epilogue is the throughput-critical part (two fp32
 // operations per output element per group), so it gets four warps per
 // scheduler; the control roles sit on two different schedulers (warp w runs
 // on scheduler w % 4) because each slows the epilogue warps that share its
@@ -295,13 +296,13 @@ constexpr uint32_t kRegsControl = 32;
 static_assert(kEpiWarps * 32 * kRegsEpilogue + 128 * kRegsControl <= kThreads * kRegsLaunch,
               "register split exceeds the launch allocation");
 constexpr uint32_t kTmemCols = 512;   // two fp32 accumulators of 256 columns
-constexpr int kRasterM = 8;
+constexpr int kRasterM = 8;  // tiles are visited in bands of 8 M-tiles
 constexpr int kRowRasterMaxN = 16;  // see tile_coords
 // Per-row scales (group_q = K): the MMA accumulates kPerRowChunk stages (256
 // of K) into one TMEM accumulator before the epilogue takes it; each such sum
 // is an integer below 256 * 112^2 < 2^22, exact in fp32 and convertible with
 // the 1.5 * 2^23 rounding addend, and the epilogue adds it to an int32.
-constexpr int kPerRowChunk = 4;           // tiles are visited in bands of 8 M-tiles
+constexpr int kPerRowChunk = 4;
 
 struct GemmArgs {
     const float *a_side;  // scales [G][m_pad], then (asymmetric) the ZeroRecs [G][m_pad]
@@ -343,11 +344,11 @@ struct GemmArgs {
 // producer writes group i + kSideSlots once the MMA of group i + kSideSlots -
 // kStages is done, which was issued after the epilogue had released group
 // i + kSideSlots - kStages - 2, a group after i.
-constexpr int kOutBlockBytes = 32 * 128;  // 32 rows of 64 two-byte outputs
 //
 // With zero points (ZERO) a stage also holds its group's records as rows of 16
 // bytes, the upper halves zero, 128 of activations and 256 of weights, and a
 // zero block stands for the second 16 bytes of K of both.
+constexpr int kOutBlockBytes = 32 * 128;  // 32 rows of 64 two-byte outputs
 constexpr int kRecRow = 16;
 constexpr int kRecBytes = (BM + BN) * kRecRow;
 template <bool ZERO, bool STAGED>

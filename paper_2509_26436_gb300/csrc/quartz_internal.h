@@ -126,7 +126,9 @@ void linear_workspace_carve(void *base, int64_t M, int64_t N, int64_t K, int mod
 cudaError_t launch_prepare(const quartz_encoded_t *a, const quartz_encoded_t *w, const LinearWorkspace &ws,
                            cudaStream_t s, bool expand = true, bool w_ready = false);
 // Layout of a prepared weight operand: the expanded operand [round_up(N, 16),
-// K] bytes, then the side values [nside][K/64][round_up(N, 256)] fp32.
+// K] bytes, then the scales [K/64][round_up(N, 256)] fp32 and, in the
+// asymmetric mode, as many 8-byte zero-point records (linear.cu, ZeroRec).
+// Made and read by the same build of the library.
 size_t prepared_weights_bytes(int64_t N, int64_t K, int mode);
 void prepared_weights_carve(const void *base, int64_t N, int64_t K, int mode, LinearWorkspace *ws);
 // The paper's accumulator-shift schedule on CUDA cores, from the packed codes;
