@@ -29,8 +29,11 @@
 //     both caches (8 KB each per 128 tokens) stream through a 2-stage
 //     shared-memory ring filled by cp.async (chunks XOR-swizzled against
 //     bank conflicts) one tile ahead (more stages measured slower: fewer
-//     CTAs fit an SM); FLAGs and scales of the next tile are prefetched
-//     into registers.  Output per CTA: unnormalised o, running
+//     CTAs fit an SM); FLAGs and scales of the next tile are loaded into the
+//     registers of this one's once these are used, before the value phase
+//     (loaded a whole tile ahead, the copies and the registers they hold cost
+//     more: G_s = 8 70.7 -> 69.2 us, 16 64.1 -> 63.1, 64 62.8 -> 59.8, 32 x 16
+//     heads, 4096 tokens).  Output per CTA: unnormalised o, running
 //     max, running sum.
 //     What bounds it: instruction issue as much as memory.  A 128-token tile
 //     took 842 instructions a warp (32 x 16 heads, 4096 tokens, G_s = 16:
@@ -351,10 +354,6 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
         __syncthreads();     // ... and everyone else's
         const uint32_t kst = ring + (it % kStages) * 2 * kTileBytes;
         const uint32_t vst = kst + kTileBytes;
-        // FLAGs and scales of the next tile, while this one is processed
-        RowSide nxt;
-        const int t_next = (it + 1) * kTile + tid;
-        load_side<GS, PACK>(a, side, static_cast<uint32_t>(t_next), t_next < n_tok, nxt);
 
         // ---- keys: one token per thread -----------------------------------
         const bool valid = it * kTile + tid < n_tok;
@@ -402,6 +401,9 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
 #pragma unroll
         for (int j = 0; j < S; ++j)  // p_t s_v 2^FLAG of every value subgroup (0 past the end)
             s_pf[j][tid] = p * scale_pow2((j * GS) / 64 ? cur.sv.y : cur.sv.x, row_flag(cur.vf, j, v_packed));
+        // FLAGs and scales of the next tile, while the values are processed
+        const int t_next = (it + 1) * kTile + tid;
+        load_side<GS, PACK>(a, side, static_cast<uint32_t>(t_next), t_next < n_tok, cur);
         if (m_new != m_run) {  // CTA-uniform: rescale only when the maximum grew
 #pragma unroll
             for (int k = 0; k < kValDims; ++k) acc[k] *= alpha;
@@ -429,7 +431,6 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
                                magic_float(od, 0x7440u | b));
             }
         }
-        cur = nxt;
         __syncthreads();  // s_pf and this stage are rewritten later
     }
     cp_async_wait<0>();
