@@ -42,11 +42,12 @@
 //     is kept small: addresses are a base per CTA plus 32-bit offsets, a full
 //     tile is copied without row checks, the FLAG form (bytes or nibbles) is a
 //     template argument, and a key's FLAG shifts the 16-fold dot product,
-//     which is divided by 16 once per 64-wide group.  72.7 -> 64.7 us there,
-//     80.7 -> 71.4 at G_s = 8, 68.4 -> 62.4 at G_s = 32 (with the value layout
-//     below), 131 -> 116 with 64 x 16 heads.  Measured and not used: independent warps without CTA barriers
-//     (+-3%); the tiles of all heads cut into equal runs, one wave of CTAs
-//     (0-8% slower).
+//     which is divided by 16 once per 64-wide group.  With what the comments
+//     below add, 72.7 -> 62.0 us there, 80.7 -> 67.6 at G_s = 8, 68.4 -> 61.7
+//     at G_s = 32, 131 -> 112 with 64 x 16 heads.  Measured and not used:
+//     independent warps without CTA barriers (+-3%); the tiles of all heads
+//     cut into equal runs, one wave of CTAs (0-8% slower); the even key codes
+//     biased in their low nibbles instead of shifted (1-3% slower).
 //   attn_combine_kernel: one CTA per bh merges the splits, where
 //     attn_decode_kernel does not do it itself (one split, or one wave of
 //     CTAs with at most 8 splits a head).
@@ -127,8 +128,8 @@ __device__ __forceinline__ float2 load_scales2(const __half *scales, Row row)
     return __half22float2(*reinterpret_cast<const __half2 *>(&w));
 }
 
-// The float 2^23 + (c + 8) for the biased code byte selected by `sel` (byte
-// b of `biased_bytes` into byte 0, 0x4B above it: 0x4B0000xx = 2^23 + xx).
+// The float 2^23 + x for the byte x selected by `sel` (byte b of
+// `biased_bytes` into byte 0, 0x4B above it: 0x4B0000xx = 2^23 + xx).
 __device__ __forceinline__ float magic_float(uint32_t biased_bytes, uint32_t sel)
 {
     return __int_as_float(prmt_b32(biased_bytes, 0x4B000000u, sel));
@@ -148,20 +149,23 @@ __device__ __forceinline__ float scale_pow2(float s, int F)
     return __int_as_float(__float_as_int(s) + (F << 23));
 }
 
-// (acc0, acc1) += p * (c0, c1), where c = f - (2^23 + 8) for the magic floats
-// f: one paired subtraction and one paired fused multiply-add.
+// (acc0, acc1) += p * (c0, 16 c1), where f0 = 2^23 + 8 + c0 and f1 = 2^23 + 16
+// (8 + c1): one paired subtraction and one paired fused multiply-add.  The
+// odd codes stay in their high nibbles, which saves a shift per 8 codes; their
+// sums are 16-fold until the end (a power of two: the roundings are the same).
+// 32 x 16 heads, 4096 tokens: G_s = 8 69.2 -> 67.5 us, 16 63.1 -> 62.0.
 __device__ __forceinline__ void fma_codes2(float &acc0, float &acc1, float p, float f0, float f1)
 {
     asm("{\n\t.reg .b64 f, m, c, pp, acc;\n\t"
         "mov.b64 f, {%2, %3};\n\t"
-        "mov.b64 m, {%5, %5};\n\t"
+        "mov.b64 m, {%5, %6};\n\t"
         "add.rn.f32x2 c, f, m;\n\t"
         "mov.b64 pp, {%4, %4};\n\t"
         "mov.b64 acc, {%0, %1};\n\t"
         "fma.rn.f32x2 acc, pp, c, acc;\n\t"
         "mov.b64 {%0, %1}, acc;\n\t}"
         : "+f"(acc0), "+f"(acc1)
-        : "f"(f0), "f"(f1), "f"(p), "f"(-8388616.0f));
+        : "f"(f0), "f"(f1), "f"(p), "f"(-8388616.0f), "f"(-8388736.0f));
 }
 
 // Asynchronous 16-byte global -> shared copies (cp.async, completion tracked
@@ -424,7 +428,7 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
                 const int sub = (kWordsPerPiece * vc + w) / kWordsPerSub;
                 const float pf = s_pf[sub][ti];
                 const uint32_t ev = (words[w] & 0x0F0F0F0Fu) ^ 0x08080808u;         // codes 0, 2, 4, 6 as c + 8
-                const uint32_t od = ((words[w] >> 4) & 0x0F0F0F0Fu) ^ 0x08080808u;  // codes 1, 3, 5, 7
+                const uint32_t od = (words[w] & 0xF0F0F0F0u) ^ 0x80808080u;  // codes 1, 3, 5, 7 as 16 (c + 8)
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
                     fma_codes2(acc[8 * w + 2 * b], acc[8 * w + 2 * b + 1], pf, magic_float(ev, 0x7440u | b),
@@ -442,7 +446,7 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
     __syncthreads();
     float *s_red = reinterpret_cast<float *>(s_ring);
 #pragma unroll
-    for (int k = 0; k < kValDims; ++k) s_red[(slot * kPieces + vc) * (kValDims + 1) + k] = acc[k];
+    for (int k = 0; k < kValDims; ++k) s_red[(slot * kPieces + vc) * (kValDims + 1) + k] = k & 1 ? acc[k] * 0.0625f : acc[k];
     float ws = l_thr;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
