@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(kAttnThreads, attn_min_ctas<GS>()) attn_decode
                     dot = __dp4a(static_cast<int>(qe[w]), static_cast<int>((kw[w] << 4) & 0xF0F0F0F0u), dot);
                     dot = __dp4a(static_cast<int>(qo[w]), static_cast<int>(kw[w] & 0xF0F0F0F0u), dot);
                 }
-                P[(j * GS) / 64] += dot << row_flag(cur.kf, j, k_packed);  // 16 x the group sum, in 27 bits
+                // 16 x the group sum, in 27 bits (the shift of a negative sum as unsigned)
+                P[(j * GS) / 64] += static_cast<int>(static_cast<uint32_t>(dot) << row_flag(cur.kf, j, k_packed));
             }
             const float sc = __fmul_rn(__fmul_rn(sq.x, cur.sk.x), static_cast<float>(P[0] >> 4)) +
                              __fmul_rn(__fmul_rn(sq.y, cur.sk.y), static_cast<float>(P[1] >> 4));
