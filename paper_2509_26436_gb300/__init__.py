@@ -58,10 +58,18 @@ class Params:
         return N.QuartzParams(self.group_q, self.group_s, self.mode, self.flag_bits, self.code_bits)
 
 
-@lru_cache(maxsize=256)
+@lru_cache(maxsize=256, typed=True)
+def _c_fields(*fields) -> N.QuartzParams:
+    """The C struct of these five fields (only ever read).  Typed: a value of
+    a type the struct refuses, equal to one it takes (64.0 and 64), is looked
+    up by itself and refused by ctypes on every call."""
+    return N.QuartzParams(*fields)
+
+
 def _c_params(params: Params) -> N.QuartzParams:
-    """The C struct of `params` (plain numbers; only ever read)."""
-    return params.c()
+    if type(params) is not Params:
+        return params.c()
+    return _c_fields(params.group_q, params.group_s, params.mode, params.flag_bits, params.code_bits)
 
 
 class Encoded:
