@@ -116,7 +116,10 @@ typedef struct {
 /* Human-readable name of a status code (static storage; never NULL). */
 const char *quartz_status_string(int32_t status);
 
-/* ABI version of this library: (major << 16) | minor. */
+/* Version of this library: (major << 16) | minor.  The minor number also
+ * counts the layouts of prepared weights (quartz_prepare_weights): a buffer
+ * made under another version may not be used.  1.8: zero-point records in
+ * place of two fp32 planes (ASYMMETRIC; the size is the same). */
 int32_t quartz_version(void);
 
 /* Bytes of each buffer of an encoded [rows, K] tensor, for allocation:
@@ -235,8 +238,12 @@ size_t quartz_prepared_weights_size(int64_t N, int64_t K, const quartz_params_t 
 
 /* Prepare encoded weights [N, K] once (offline, like their encoding): their
  * tensor-core operand (the decoded values, E4M3, or E5M2 for 16-bit codes)
- * and transposed group scales, written to `prepared` (device memory owned by
- * the caller, >= quartz_prepared_weights_size bytes, 16-byte aligned).  A
+ * and transposed group scales (ASYMMETRIC: and zero-point terms), written to
+ * `prepared` (device memory owned by the caller, >=
+ * quartz_prepared_weights_size bytes, 16-byte aligned).  The layout is private
+ * to the version that wrote it: a program that stores the buffer stores
+ * quartz_version() with it and prepares again when that differs, since a
+ * buffer of another layout passes every check and gives wrong results.  A
  * later quartz_linear_ex with opts->w_prepared = prepared and the same `w`
  * skips that work on every call; the buffer is only valid for that `w`
  * (its codes, FLAGs, scales and params) and becomes stale if `w` changes. */

@@ -212,7 +212,8 @@ def _out_type(dtype) -> int:
 
 def prepare_weights(w: Encoded, stream=None):
     """The weights' tensor-core operand and scale side values, prepared once
-    (offline, like the encoding) for linear(..., w_prepared=...)."""
+    (offline, like the encoding) for linear(..., w_prepared=...).  A buffer
+    that is stored is only good for the quartz_version() that made it."""
     torch = _torch()
     n = N.load().quartz_prepared_weights_size(w.rows, w.K, _byref(_c_params(w.params)))
     if n == 0:

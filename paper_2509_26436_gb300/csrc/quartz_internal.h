@@ -128,7 +128,8 @@ cudaError_t launch_prepare(const quartz_encoded_t *a, const quartz_encoded_t *w,
 // Layout of a prepared weight operand: the expanded operand [round_up(N, 16),
 // K] bytes, then the scales [K/64][round_up(N, 256)] fp32 and, in the
 // asymmetric mode, as many 8-byte zero-point records (linear.cu, ZeroRec).
-// Made and read by the same build of the library.
+// A change here raises quartz_version(): stored buffers carry no mark of
+// their own (quartz.h).
 size_t prepared_weights_bytes(int64_t N, int64_t K, int mode);
 void prepared_weights_carve(const void *base, int64_t N, int64_t K, int mode, LinearWorkspace *ws);
 // The paper's accumulator-shift schedule on CUDA cores, from the packed codes;
