@@ -524,35 +524,66 @@ __global__ void __launch_bounds__(kD) attn_combine_kernel(const float *__restric
     const int64_t bh = blockIdx.x;
     const int d = threadIdx.x;
     const float *p = part + bh * n_split * kPartStride;
-    // The kernel is all latency.  The first 8 splits' values are loaded
+    // The kernel is all latency.  Up to 8 splits: their values are loaded
     // together, not maxima first: 32 x 4 heads with 8 splits 19.6 -> 18.6 us
     // for the whole step, 32 x 16 heads with 4 splits 64.6 -> 64.1; 4 or 16
     // instead of 8 measured within 0.3 us at 4 splits, and 4 costs 0.7 at 8.
     constexpr int kCombine = 8;
-    float m[kCombine], l[kCombine], o[kCombine];
-#pragma unroll
-    for (int s = 0; s < kCombine; ++s) {
-        const bool in = s < n_split;
-        m[s] = in ? p[s * kPartStride + kD] : -INFINITY;
-        l[s] = in ? p[s * kPartStride + kD + 1] : 0.f;
-        o[s] = in ? p[s * kPartStride + d] : 0.f;
-    }
-    float M = -INFINITY;
-#pragma unroll
-    for (int s = 0; s < kCombine; ++s) M = fmaxf(M, m[s]);
-    for (int s = kCombine; s < n_split; ++s) M = fmaxf(M, p[s * kPartStride + kD]);
     float num = 0.f, den = 0.f;
+    if (n_split <= kCombine) {
+        float m[kCombine], l[kCombine], o[kCombine];
+        float M = -INFINITY;
 #pragma unroll
-    for (int s = 0; s < kCombine; ++s)
-        if (s < n_split) {
-            const float w = exp2f(m[s] - M);  // 0 for an empty split
-            num = fmaf(w, o[s], num);
-            den = fmaf(w, l[s], den);
+        for (int s = 0; s < kCombine; ++s) {
+            const bool in = s < n_split;
+            m[s] = in ? p[s * kPartStride + kD] : -INFINITY;
+            l[s] = in ? p[s * kPartStride + kD + 1] : 0.f;
+            o[s] = in ? p[s * kPartStride + d] : 0.f;
         }
-    for (int s = kCombine; s < n_split; ++s) {
-        const float w = exp2f(p[s * kPartStride + kD] - M);
-        num = fmaf(w, p[s * kPartStride + d], num);
-        den = fmaf(w, p[s * kPartStride + kD + 1], den);
+#pragma unroll
+        for (int s = 0; s < kCombine; ++s) M = fmaxf(M, m[s]);
+#pragma unroll
+        for (int s = 0; s < kCombine; ++s)
+            if (s < n_split) {
+                const float w = exp2f(m[s] - M);  // 0 for an empty split
+                num = fmaf(w, o[s], num);
+                den = fmaf(w, l[s], den);
+            }
+    } else {
+        // More (few heads): thread s loads split s's maximum and sum and
+        // computes its weight once, and the outputs come kBatch splits at a
+        // time, the first of them before the weights are known.  Same
+        // arithmetic in the same order.  A loop over the splits in every
+        // thread, its loads one after the other, cost more than the step: 3
+        // heads, 8097 tokens (64 splits), G_s = 8 14.6 -> 7.1 us; 15 heads,
+        // 7534 tokens (59 splits), G_s = 64 13.8 -> 9.2.
+        constexpr int kBatch = 16;
+        static_assert(kMaxSplits == 64 && kD >= kMaxSplits, "two maxima per lane, a thread per split");
+        __shared__ float s_m[kMaxSplits], s_w[kMaxSplits], s_l[kMaxSplits];
+        float o[kBatch];
+        auto load_o = [&](int s0) {
+#pragma unroll
+            for (int s = 0; s < kBatch; ++s) o[s] = s0 + s < n_split ? p[(s0 + s) * kPartStride + d] : 0.f;
+        };
+        load_o(0);
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (d < n_split) ml = *reinterpret_cast<const float2 *>(p + d * kPartStride + kD);
+        if (d < kMaxSplits) s_m[d] = ml.x, s_l[d] = ml.y;
+        __syncthreads();
+        float M = fmaxf(s_m[d & 31], s_m[32 + (d & 31)]);
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, k));
+        if (d < n_split) s_w[d] = exp2f(ml.x - M);  // 0 for an empty split
+        __syncthreads();
+        for (int s0 = 0; s0 < n_split; s0 += kBatch) {
+            if (s0 > 0) load_o(s0);
+#pragma unroll
+            for (int s = 0; s < kBatch; ++s)
+                if (s0 + s < n_split) {
+                    num = fmaf(s_w[s0 + s], o[s], num);
+                    den = fmaf(s_w[s0 + s], s_l[s0 + s], den);
+                }
+        }
     }
     store_out(out, OUT, bh * kD + d, num / den);
 }
