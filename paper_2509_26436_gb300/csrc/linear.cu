@@ -660,6 +660,53 @@ __device__ __forceinline__ void lds_b64x2(uint32_t addr, uint64_t &a, uint64_t &
     asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
 
+// Partials dump: one epilogue warp's 32 x 64 slice (first row m0, first column
+// n0) of group args.partials_group, read again from its accumulator at tbase.
+// The exact integer P_g: with zero points (ZERO) the terms that the tensor core
+// added are taken off again (all integers below 2^24, exact in fp32).  It runs
+// for one group of a tile, beside the group loop that every call has.  Against a
+// group loop of its own that fetched the zero points per group from global
+// memory (GEMM 4001 x 3456 x 1152, fp16 / fp32 out): 203 -> 60 / 166 -> 64 us
+// with zero points (37.5 / 44 without a dump), 85 -> 44 / 89 -> 52 without
+// (33 / 40).
+template <bool ZERO>
+__device__ __forceinline__ void dump_partials(const GemmArgs &args, uint32_t tbase, int64_t m0, int64_t n0)
+{
+    int lane;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+    m0 += lane >> 2;
+    n0 += 4 * (lane & 3);
+    const int64_t g = args.partials_group;
+#pragma unroll 1
+    for (int chunk = 0; chunk < 4; ++chunk, n0 += 16) {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            uint32_t r[8];  // columns n0 + i of rows m0 + 16 h (r[2 i]) and 8 below (r[2 i + 1])
+            __syncwarp();
+            tmem_ld_16x128b_x4(tbase + (static_cast<uint32_t>(16 * h) << 16) + 16 * chunk, r);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int64_t m = m0 + 16 * h + 8 * e;
+                float2 ta = make_float2(0.f, 0.f);
+                if (ZERO) ta = zero_terms(zero_recs(args.a_side, args.G, args.m_pad)[g * args.m_pad + m], true);
+                int32_t P[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float p = __uint_as_float(r[2 * i + e]);
+                    if (ZERO) {
+                        const float2 tw = zero_terms(
+                            zero_recs(args.w_side, args.G, args.n_pad)[g * args.n_pad + perm16(n0 + i)], false);
+                        p = __fmaf_rn(ta.x, tw.y, __fmaf_rn(-tw.x, ta.y, p));
+                    }
+                    P[i] = __float2int_rn(p);
+                }
+                if (m < args.M && n0 < args.N)
+                    *reinterpret_cast<int4 *>(args.partials + m * args.N + n0) = make_int4(P[0], P[1], P[2], P[3]);
+            }
+        }
+    }
+}
+
 template <int MODE, int OUT, bool DUMP, bool PERROW, int RM = kRasterM>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a,
@@ -667,7 +714,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const GemmArgs args)
 {
     griddep_wait();
-    constexpr bool ZERO = MODE == QUARTZ_ASYMMETRIC && !DUMP;  // zero-point terms by the tensor core
+    constexpr bool ZERO = MODE == QUARTZ_ASYMMETRIC;  // zero-point terms by the tensor core
     using L = Smem<ZERO, OUT != QUARTZ_OUT_F32>;
     constexpr int kStages = L::kStages, kStageBytes = L::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -998,8 +1045,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 out.end();
             }
-        } else if constexpr (!DUMP) {
-            // Fast path (with zero points the accumulator holds the corrected
+        } else {
+            // Groups of 64 (with zero points the accumulator holds the corrected
             // sum): each half chunk (16 lanes x 16 columns: TMEM
             // load, wait and the scale arithmetic) is one PTX block on
             // explicit 64-bit pairs, which keeps the kernel free of spills.
@@ -1046,6 +1093,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                         epi_half_chunk_sym(tbase + 16 * chunk, sw, sa0, acc64[chunk]);
                         epi_half_chunk_sym(tbase + (16u << 16) + 16 * chunk, sw, sa1, acc64[chunk] + 4);
                     }
+                    if (DUMP && left == G - args.partials_group) {  // (whole tiles: left counts down from G)
+                        int mt, nt;
+                        tile_coords<RM>(blockIdx.x + k * gridDim.x, args, mt, nt);
+                        dump_partials<ZERO>(args, tbase, static_cast<int64_t>(mt) * BM + quarter * 32,
+                                            static_cast<int64_t>(nt) * BN + slot * kColsPerWarp);
+                    }
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(full + 16);
@@ -1057,7 +1110,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
                 asm volatile("" : "+r"(k));  // the item is looked up again rather than carried through the loop
                 const WorkItem wi = work_item(args, k);
-                if (wi.part >= 0) {
+                if (!DUMP && wi.part >= 0) {
                     // split last wave: leave this part's fp32 partial tile for
                     // tail_combine_kernel: slot tail * split + part holds 16
                     // planes of one uint4 per epilogue thread (coalesced)
@@ -1111,101 +1164,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 vv[i] = __uint_as_float(static_cast<uint32_t>(e ? (q >> 32) : q));
                             }
                             out.put_raw(16 * h + 8 * e, chunk, make_float4(vv[0], vv[1], vv[2], vv[3]));
-                        }
-                out.end();
-            }
-        } else {
-            // Partials dump: raw P_g, zero-point terms from global memory.
-            float2 acc[2][16];
-            int it = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < args.num_tiles && ok; tile += gridDim.x) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[h][j] = make_float2(0.f, 0.f);
-                for (int g = 0; g < G; ++g, ++it) {
-                    const int b = it & 1;
-                    const int ss = it % L::kSideSlots;
-                    const uint32_t side_a = smem_base + L::kSide + ss * L::kSideSlotBytes + (quarter * 32 + 4 * trow) * 4;
-                    const uint32_t side_w = smem_base + L::kSide + ss * L::kSideSlotBytes + L::kSideABytes +
-                                            (slot * kColsPerWarp + tq) * 4;
-                    if (!mbar_wait_warp(acc_full_bar(b), (it >> 1) & 1, abort_flag, args.dev_err, kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
-                    int mt, nt;
-                    tile_coords<RM>(tile, args, mt, nt);
-                    const int64_t m0 = static_cast<int64_t>(mt) * BM + quarter * 32 + trow;
-                    const int64_t n0 = static_cast<int64_t>(nt) * BN + slot * kColsPerWarp + tq;
-                    const float4 sav = lds_f4(side_a);  // scales of rows trow + 8k of the quarter
-                    const float cur_a[4] = {sav.x, sav.y, sav.z, sav.w};
-                    float2 za_u[4];  // (z_a, 64 z_a - A_g) of the same rows
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        za_u[k] = MODE == QUARTZ_ASYMMETRIC
-                                      ? zero_terms(zero_recs(args.a_side, G, args.m_pad)[g * args.m_pad + m0 + 8 * k], true)
-                                      : make_float2(0.f, 0.f);
-                    tc_fence_after();
-                    const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
-                                           static_cast<uint32_t>(b * BN + slot * kColsPerWarp);
-#pragma unroll
-                    for (int chunk = 0; chunk < 4; ++chunk) {    // 16-column chunks of the slice
-                        uint32_t r[16];
-                        tmem_ld_16x128b_x4_pair(tbase + 16 * chunk, tbase + (16u << 16) + 16 * chunk, r);
-                        tmem_wait_ld(r);
-                        const float4 sw = lds_f4(side_w + 16 * chunk * 4);
-                        const float swv[4] = {sw.x, sw.y, sw.z, sw.w};
-                        float2 zg[4];  // (z_w, W_g) of the four columns
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            zg[i] = MODE == QUARTZ_ASYMMETRIC
-                                        ? zero_terms(zero_recs(args.w_side, G, args.n_pad)[g * args.n_pad + perm16(n0 + 16 * chunk + i)], false)
-                                        : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                float2 p = make_float2(__uint_as_float(r[8 * h + 2 * i]), __uint_as_float(r[8 * h + 2 * i + 1]));
-                                if (DUMP && g == args.partials_group) {
-                                    const int64_t m = m0 + 16 * h, n = n0 + 16 * chunk + i;
-                                    if (n < args.N) {
-                                        if (m < args.M) args.partials[m * args.N + n] = __float2int_rn(p.x);
-                                        if (m + 8 < args.M) args.partials[(m + 8) * args.N + n] = __float2int_rn(p.y);
-                                    }
-                                }
-                                if (MODE == QUARTZ_ASYMMETRIC) {
-                                    const float2 ua = make_float2(za_u[2 * h].y, za_u[2 * h + 1].y);
-                                    const float2 nza = make_float2(-za_u[2 * h].x, -za_u[2 * h + 1].x);
-                                    p = __ffma2_rn(make_float2(zg[i].x, zg[i].x), ua, p);
-                                    p = __ffma2_rn(nza, make_float2(zg[i].y, zg[i].y), p);
-                                }
-                                const float2 t = __fmul2_rn(p, make_float2(swv[i], swv[i]));
-                                acc[h][4 * chunk + i] = __ffma2_rn(t, make_float2(cur_a[2 * h], cur_a[2 * h + 1]),
-                                                                   acc[h][4 * chunk + i]);
-                            }
-                        }
-                    }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(acc_empty_bar(b));
-                }
-                if (!ok) break;
-                int mt, nt;
-                tile_coords<RM>(tile, args, mt, nt);
-                // ---- store: 4 rows x 4 chunks of 4 consecutive columns per thread ----
-                TileOut<OUT> out(args, &tmap_y, smem_base + L::kOut, warp, static_cast<int64_t>(mt) * BM + quarter * 32,
-                                 static_cast<int64_t>(nt) * BN + slot * kColsPerWarp);
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e)
-#pragma unroll
-                        for (int chunk = 0; chunk < 4; ++chunk) {
-                            const float2 *q = &acc[h][4 * chunk];
-                            out.put(16 * h + 8 * e, chunk,
-                                    e ? make_float4(q[0].y, q[1].y, q[2].y, q[3].y)
-                                      : make_float4(q[0].x, q[1].x, q[2].x, q[3].x));
                         }
                 out.end();
             }
@@ -1543,9 +1501,8 @@ cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tw, const CUtens
                       cudaStream_t s)
 {
     constexpr bool staged = OUT != QUARTZ_OUT_F32;
-    static_assert(Smem<true, staged>::kAlloc <= 227 * 1024 && Smem<false, staged>::kAlloc <= 227 * 1024,
-                  "shared memory budget");
-    const int smem = MODE == QUARTZ_ASYMMETRIC && !args.partials ? Smem<true, staged>::kAlloc : Smem<false, staged>::kAlloc;
+    constexpr int smem = Smem<MODE == QUARTZ_ASYMMETRIC, staged>::kAlloc;
+    static_assert(smem <= 227 * 1024, "shared memory budget");
     auto kern = args.partials ? gemm_tcgen05_kernel<MODE, OUT, true, false>
                               : gemm_tcgen05_kernel<MODE, OUT, false, false>;
     if constexpr (MODE == QUARTZ_SYMMETRIC) {
