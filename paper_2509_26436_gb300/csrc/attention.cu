@@ -57,6 +57,7 @@
 #include <atomic>
 
 #include "lzs_e4m3.cuh"
+#include "ptx.cuh"
 #include "quartz_internal.h"
 
 namespace quartz {
@@ -174,9 +175,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Shared-memory offset of 16-byte chunk c (0..3) of token row r in a code
 // tile: rows of 64 bytes, chunks XOR-swizzled by (r / 2) % 4 so that eight

@@ -7,8 +7,9 @@
 //      at most 3 significant bits and |v| <= 112, inside E4M3's 4-bit
 //      significand and 448 range), together with the group scales
 //      transposed to [G][rows] fp32 (and the zero-point terms to records in
-//      the same order, see ZeroRec) for contiguous per-group access.  This pass is HBM-bound and touches each operand
-//      element once, instead of once per output tile that reads it.
+//      the same order, see ZeroRec) for contiguous per-group access.  This
+//      pass is HBM-bound and touches each operand element once, instead of
+//      once per output tile that reads it.
 //   2. GEMM: a persistent warp-specialised tcgen05 kernel.  One TMA warp
 //      streams 128x64 A and 256x64 W tiles (one 64-wide quantization group
 //      per stage, 64-byte swizzle) into a 5-stage shared-memory ring, with
@@ -61,15 +62,6 @@ __host__ __device__ __forceinline__ int64_t perm16(int64_t r)
     return (r & ~int64_t(15)) | ((r & 3) << 2) | ((r >> 2) & 3);
 }
 
-// One launch prepares both GEMM operands (jobs selected by block index):
-//   expand A, expand W: 16 codes per thread (8 bytes in, 16 E4M3 bytes out);
-//     the weight operand is row-permuted (perm16) and zero-padded to a
-//     multiple of 16 rows;
-//   side A, side W: side[0][g][.] = s[r, g], weight rows in natural order,
-//     activation rows at perm32(r); asymmetric adds a ZeroRec per row and
-//     group (see there) in the space of two more such planes.  Rows in
-//     [rows, rows_pad) are 0.  One thread per row and 8 groups: its reads stay
-//     in L1 lines, consecutive threads write consecutive rows.
 // Zero-point terms of one row and group.  With u = 64 z_a - A_g (A_g, W_g: the
 // gsum side values) the integer correction is P + z_w u - z_a W_g, the dot
 // product of an activation record (hi u, lo u, -z_a, -z_a) and a weight
@@ -113,6 +105,15 @@ __host__ __device__ __forceinline__ const ZeroRec *zero_recs(const float *side, 
     return reinterpret_cast<const ZeroRec *>(side + G * rows_pad);
 }
 
+// One launch prepares both GEMM operands (jobs selected by block index):
+//   expand A, expand W: 16 codes per thread (8 bytes in, 16 E4M3 bytes out);
+//     the weight operand is row-permuted (perm16) and zero-padded to a
+//     multiple of 16 rows;
+//   side A, side W: side[0][g][.] = s[r, g], weight rows in natural order,
+//     activation rows at perm32(r); asymmetric adds a ZeroRec per row and
+//     group (see there) in the space of two more such planes.  Rows in
+//     [rows, rows_pad) are 0.  One thread per row and 8 groups: its reads stay
+//     in L1 lines, consecutive threads write consecutive rows.
 struct ExpandJob {
     const uint2 *codes;          // [rows, K/16] units of 16 codes
     const uint8_t *flags;        // [rows, K/G_s]
@@ -322,8 +323,9 @@ struct GemmArgs {
     // Split last wave: the first full_tiles tiles go round robin over the CTAs
     // (the same count each); each of the remaining tail_tiles is cut along K
     // into `split` group ranges taken by CTAs 0 .. tail_tiles * split - 1,
-    // which leave fp32 partial tiles in tail_part; tail_combine_kernel adds
-    // them in part order and writes the outputs.  Range forms (ls > 0): the
+    // which leave partial tiles in tail_part (fp32 sums, or int32 sums with
+    // scales per row); tail_combine_kernel adds them in part order and writes
+    // the outputs.  Range forms (ls > 0): the
     // last tail_tiles tiles' tail_tiles * G group iterations (after at least
     // one wave of whole tiles, or every tile's when more than half but not
     // all of the SMs hold one) are cut into one contiguous range of ls per
@@ -332,7 +334,7 @@ struct GemmArgs {
     // where ls >= G / 2), a tile inside one range is stored whole.
     int full_tiles, tail_tiles, split;
     int ls;
-    float *tail_part;     // [tail_tiles][split][16][kEpiWarps * 32] float4 (fp32 pairs)
+    float *tail_part;     // [tail_tiles][split][16][kEpiWarps * 32] of four 32-bit words (fp32, or int32 per row)
 };
 
 // Shared memory: the operand stages, the output blocks (one per epilogue warp,
@@ -1053,10 +1055,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             // The group loop carries only its accumulators, three offsets and
             // a count: with the work item and a group index carried too, ptxas
             // spilled and added moves (18432 x 12288 x 3072 1047 us, now 984;
-            // 8192 x 4608 x 1152 84.6, now 79; both with TileOut).  It runs at
-            // about 0.85 of what the pair operations alone take: mul + fma on
-            // f32x2 pairs with distinct operands need 5.5 cycles a pair and
-            // scheduler (register reads), 704 per group of a tile.  Loads of
+            // 8192 x 4608 x 1152 84.6, now 79; both with TileOut).  A group takes
+            // 850 cycles (18432 x 12288 x 3072, ends of tiles included) against
+            // 512 of fp32 lanes: FMA pipe 64% busy, issue slots 65%.  Loads of
             // 32 columns or of both lane halves per wait, and scales loaded
             // ahead, measured 1-10% slower.
             // acc64[c][4h + i]: output column 16c + tq + i, rows trow + 16h (low) and + 8 (high)
@@ -1179,9 +1180,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-// Split last wave (see GemmArgs): adds each tail tile's `split` fp32
-// partial tiles in part order, then stores the sum as the epilogue would
-// have.  Grid: (tail tile, 16-column chunk c of every warp's slice); block:
+// Split last wave (see GemmArgs): adds each tail tile's partial tiles in part
+// order (fp32, or int32 with scales per row, which are then applied), then
+// stores the sum as the epilogue would have.  Grid: (tail tile, 16-column chunk c of every warp's slice); block:
 // one thread per epilogue thread, which owns the chunk's 8 column pairs.
 template <int OUT, bool PERROW>
 __global__ void __launch_bounds__(kEpiWarps * 32) tail_combine_kernel(const __grid_constant__ GemmArgs args)
@@ -1618,8 +1619,8 @@ GemmArgs make_args(const LinearWorkspace &ws, int64_t M, int64_t N, int64_t K, c
 
 }  // namespace
 
-// Split of the GEMM's last wave on this device (symmetric, group-64 fast
-// path): when the tiles left after whole waves fill at most half of one,
+// Split of the GEMM's last wave on this device (symmetric mode; with scales per
+// row row_split_pays decides whether it is taken): when the tiles left after whole waves fill at most half of one,
 // each of them is cut along K into `split` group ranges (at most
 // kMaxTailSplit, at least two groups each) for otherwise idle CTAs; with
 // fewer tiles than SMs (a first wave that is also the last), every tile is

@@ -84,10 +84,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// Bounded wait on an mbarrier phase.  Gives up after `limit_ns` of wall time
-// or as soon as another role of the CTA has raised `abort_flag`; on a timeout
-// it raises the CTA's abort flag and records QUARTZ_DEV_TIMEOUT in the
-// library's device error word `dev_err`.  Returns true iff the phase completed.
 // try_wait that may suspend the thread in hardware until the phase completes
 // or `hint_ns` elapses, so waiting threads do not take issue slots.
 __device__ __forceinline__ bool mbar_try_wait_sleep(uint32_t bar, uint32_t parity, uint32_t hint_ns)
@@ -103,6 +99,10 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(uint32_t bar, uint32_t parit
     return ok != 0;
 }
 
+// Bounded wait on an mbarrier phase.  Gives up after `limit_ns` of wall time
+// or as soon as another role of the CTA has raised `abort_flag`; on a timeout
+// it raises the CTA's abort flag and records QUARTZ_DEV_TIMEOUT in the
+// library's device error word `dev_err`.  Returns true iff the phase completed.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
                                                   volatile int *abort_flag, int *dev_err,
                                                   uint64_t limit_ns)

@@ -104,11 +104,11 @@ struct LinearWorkspace {
     void *w_op;      // E4M3 [round_up(N, 16), K]  decoded weights, rows transposed 4x4 inside 16-row blocks
     float *a_side;   // fp32 [G][Mpad] scales; asymmetric: then 8-byte zero-point records [G][Mpad] (linear.cu: ZeroRec)
     float *w_side;   // the same [G][Npad]
-    float *tail_part;  // fp32 partial tiles of the split last wave (may be NULL)
+    float *tail_part;  // partial tiles of the split last wave: fp32, or int32 with scales per row (may be NULL)
     int64_t m_pad, n_pad;
     int nside;
     int tail_tiles, tail_split;  // tiles of the split last wave(s) and parts per tile (1 = no split)
-    int tail_ls;                 // two-wave form: group iterations per CTA (0: one-wave form)
+    int tail_ls;                 // range forms (two waves, or fewer tiles than SMs): group iterations per CTA (0: equal parts)
 };
 size_t linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int mode);
 // Parts each tile of the symmetric tcgen05 GEMM's split last wave is cut
