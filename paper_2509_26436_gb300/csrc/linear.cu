@@ -1282,7 +1282,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const __nv_fp8_e4m3 *__r
             sa[r][k] = (m0 + r < args.M) ? static_cast<int16_t>(static_cast<float>(a_op[(int64_t)(m0 + r) * K + kk])) : 0;
             sw[r][k] = (n0 + r < args.N) ? static_cast<int16_t>(static_cast<float>(w_op[perm16(n0 + r) * K + kk])) : 0;
         }
-        if (MODE == QUARTZ_ASYMMETRIC) stage_zero_terms(args, g, m0, n0, z);
+        if constexpr (MODE == QUARTZ_ASYMMETRIC) stage_zero_terms(args, g, m0, n0, z);
         __syncthreads();
         int p[4][4] = {};
         for (int k = 0; k < kGroupQ; ++k)
@@ -1300,7 +1300,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const __nv_fp8_e4m3 *__r
                 if (m >= args.M || n >= args.N) continue;
                 float P = static_cast<float>(p[i][j]);
                 if (args.partials && g == args.partials_group) args.partials[(int64_t)m * args.N + n] = p[i][j];
-                if (MODE == QUARTZ_ASYMMETRIC) {
+                if constexpr (MODE == QUARTZ_ASYMMETRIC) {
                     const float2 ta = z[0][ty * 4 + i], tw = z[1][16 * j + tx];
                     P = __fmaf_rn(tw.x, ta.y, P);
                     P = __fmaf_rn(-ta.x, tw.y, P);
@@ -1377,7 +1377,7 @@ __global__ void __launch_bounds__(256) gemm_shift_kernel(const uint32_t *__restr
             fa[r][j] = (m0 + r < args.M) ? load_flag(a_flags, (m0 + r) * flags_per_row + col, a_packed != 0) : 0;
             fw[r][j] = (n0 + r < args.N) ? load_flag(w_flags, (n0 + r) * flags_per_row + col, w_packed != 0) : 0;
         }
-        if (MODE == QUARTZ_ASYMMETRIC) stage_zero_terms(args, g, m0, n0, z);
+        if constexpr (MODE == QUARTZ_ASYMMETRIC) stage_zero_terms(args, g, m0, n0, z);
         __syncthreads();
         using Acc = typename std::conditional<WIDE, long long, int>::type;
         Acc p[4][4] = {};
@@ -1396,8 +1396,10 @@ __global__ void __launch_bounds__(256) gemm_shift_kernel(const uint32_t *__restr
                 }
         }
         float2 tws[4];
+        if constexpr (MODE == QUARTZ_ASYMMETRIC) {
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) tws[jj] = MODE == QUARTZ_ASYMMETRIC ? z[1][16 * jj + tx] : make_float2(0.f, 0.f);
+            for (int jj = 0; jj < 4; ++jj) tws[jj] = z[1][16 * jj + tx];
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int m = m0 + ty * 4 + i;
@@ -1410,7 +1412,7 @@ __global__ void __launch_bounds__(256) gemm_shift_kernel(const uint32_t *__restr
                 float P = static_cast<float>(p[i][jj]);
                 if (!WIDE && args.partials && g == args.partials_group)
                     args.partials[(int64_t)m * args.N + n] = static_cast<int32_t>(p[i][jj]);
-                if (MODE == QUARTZ_ASYMMETRIC) {
+                if constexpr (MODE == QUARTZ_ASYMMETRIC) {
                     const float2 ta = z[0][ty * 4 + i], tw = tws[jj];
                     P = __fmaf_rn(tw.x, ta.y, P);
                     P = __fmaf_rn(-ta.x, tw.y, P);
